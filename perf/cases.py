@@ -472,7 +472,8 @@ def work(case):
 
 
 def tolerance(case):
-    return {"rel": 1e-4} if case["dtype"] == "f32" else {"rel": 1e-12}
+    # errors against `exact` reach 1e-6 and 3e-15; a few lanes whose gradient cancels show more
+    return {"rel": 4e-5} if case["dtype"] == "f32" else {"rel": 2e-13}
 
 
 # --------------------------------------------------------------------------- 64-bit answers
