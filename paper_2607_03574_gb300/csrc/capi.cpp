@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "compact.h"
 #include "plan.h"
 #include "replay.h"
 #include "status.h"
@@ -37,6 +38,7 @@ ndvm_status cuda_fail(cudaError_t e, const char* where) {
 struct DevPlan {
   std::vector<DevPlan> derive;  // derive plans of the shared per-point values
   DInst* code = nullptr;
+  DInst* compact = nullptr;      // the compact records, or null
   DInst* code_paired = nullptr;  // the paired stream (staged and element-split variants), or null
   int32_t* args = nullptr;
   double* consts_d = nullptr;
@@ -68,7 +70,7 @@ namespace {
 
 void free_plan(DevPlan& p) {
   for (DevPlan& d : p.derive) free_plan(d);
-  cudaFree(p.code); cudaFree(p.code_paired); cudaFree(p.args); cudaFree(p.consts_d); cudaFree(p.consts_f);
+  cudaFree(p.code); cudaFree(p.compact); cudaFree(p.code_paired); cudaFree(p.args); cudaFree(p.consts_d); cudaFree(p.consts_f);
   p = DevPlan{};
 }
 
@@ -90,6 +92,13 @@ ndvm_status upload_plan(const Tape& t, const Plan& p, DevPlan& d) {
   if (!p.code_paired.empty()) {
     if ((e = cudaMalloc(&d.code_paired, sizeof(DInst) * (p.code_paired.size() + 1))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = cudaMemcpy(d.code_paired, p.code_paired.data(), sizeof(DInst) * p.code_paired.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+      return cuda_fail(e, "cudaMemcpy");
+  }
+  if (!p.compact.empty()) {
+    void* c = nullptr;
+    if ((e = cudaMalloc(&c, sizeof(uint32_t) * p.compact.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    d.compact = static_cast<DInst*>(c);
+    if ((e = cudaMemcpy(c, p.compact.data(), sizeof(uint32_t) * p.compact.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
       return cuda_fail(e, "cudaMemcpy");
   }
   d.derive.resize(p.derive.size());
@@ -187,6 +196,8 @@ bool stage_enabled() {
 struct Shape {
   int tpb = 128, log2g = 0, shared = 0, sstride = 128;
   int staged = 0, stage_off = 0;
+  int points = 0;  // compact stream: points per thread and pass (0: the general kernels)
+  int chunk_lanes = 0;  // lanes that a launch over part of the lanes is a multiple of
   size_t smem = 0;
 };
 
@@ -196,7 +207,58 @@ int ilog2(int g) {
   return l;
 }
 
-Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
+// The launch shape of a compact stream; false when it does not fit.  Threads per lane and
+// points per thread depend on the lanes and the points alone, so that a tape's value and
+// gradient plans sum in the same order.
+bool compact_shape(const Plan& p, size_t elem, int64_t B, Shape* out) {
+  if (p.compact.empty()) return false;
+  Shape s;
+  const int64_t sms = num_sms();
+  const size_t records = p.compact.size() / kCompactWords;
+  const bool axis = p.compact_points > 0;
+  // up to kCResident records are held in shared memory whole; longer streams are read in
+  // chunks, which loops do not allow (the general kernels run those)
+  const bool chunked = records > kCResident;
+  if (chunked && axis) return false;
+  s.points = 1;
+  if (axis && p.n_save == 0) {
+    int g = threads_per_lane_override();
+    if (!g) {
+      g = 1;
+      while (g < 32 && B * g < sms * 192) g *= 2;
+    }
+    s.log2g = ilog2(g);
+    if (p.compact_points > g) s.points = elem == 4 ? kPointsF32 : kPointsF64;
+  }
+  s.staged = chunked ? 1 : 0;
+  s.sstride = p.compact_slots;
+  s.stage_off = (int)(((chunked ? 2 * kCChunk : records) + 3) * kCompactWords * 4);  // (records are read ahead)
+  const size_t warp_bytes = (size_t)p.compact_slots * 32 * s.points * elem;
+  const int64_t warps = ((B << s.log2g) + 31) / 32;
+  // threads per block: the most warps per SM at a time, then the fewest on the busiest SM
+  int best_res = 0;
+  int64_t best_busy = 0;
+  for (int t = 128; t >= 32; t /= 2) {
+    const int w = t / 32;
+    const size_t smem = (size_t)s.stage_off + w * warp_bytes;
+    if (smem > kSmemLimit) continue;
+    const int blocks = std::min<int>((int)(kSmemPerSm / (smem + kSmemPerBlockReserved)), kRegsPerSm / (kMaxRegsStagedOrShared * t));
+    const int64_t grid = (warps + w - 1) / w;
+    const int64_t busy = (grid + sms - 1) / sms * w;
+    const int res = (int)std::min<int64_t>((int64_t)blocks * w, busy);
+    if (best_res == 0 || (busy > res ? res > best_res : best_res < best_busy ? res > best_res : busy < best_busy)) {
+      best_res = res;
+      best_busy = busy;
+      s.tpb = t;
+      s.smem = smem;
+    }
+  }
+  if (best_res == 0) return false;
+  *out = s;
+  return true;
+}
+
+Shape general_shape(const Plan& p, size_t elem, int64_t B) {
   Shape s;
   const int64_t sms = num_sms();
   const int ov = threads_per_lane_override();
@@ -272,6 +334,36 @@ Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
   return s;
 }
 
+// A replay's arguments that its plan, launch shape and type decide.
+void plan_args(ReplayArgs& a, const Plan& p, const DevPlan& d, const Shape& sh, ndvm_dtype dtype, int* err) {
+  // the staged and element-split variants run the paired stream; the plain one does not
+  // carry the paired instruction (it would cost its register budget)
+  const bool paired = (sh.staged || sh.shared) && d.code_paired != nullptr;
+  a.code = sh.points ? d.compact : paired ? d.code_paired : d.code;
+  a.n_code = (int)(sh.points ? p.compact.size() / kCompactWords : paired ? p.code_paired.size() : p.code.size());
+  a.args = d.args;
+  a.consts = dtype == NDVM_F32 ? (const void*)d.consts_f : (const void*)d.consts_d;
+  a.P = p.n_params;
+  a.log2g = (int16_t)sh.log2g;
+  a.shared_lane = (int16_t)sh.shared;
+  a.sstride = sh.sstride;
+  a.staged = (int16_t)sh.staged;
+  a.stage_off = sh.stage_off;
+  a.points = (int16_t)sh.points;
+  a.err = err;
+}
+
+// A partial launch (a workspace smaller than all lanes need) covers a multiple of the general
+// kernels' lanes per block, whichever kernel runs: the smallest workspace a call accepts
+// depends on the tape and its lanes only.
+Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
+  const Shape g = general_shape(p, elem, B);
+  Shape s = g;
+  if (!compact_shape(p, elem, B, &s)) s = g;
+  s.chunk_lanes = g.tpb >> g.log2g;
+  return s;
+}
+
 // bytes of the extended observations (a copy of the observations the program reads,
 // then the regions' blocks of shared per-point values), rounded up to 256; 0 without
 size_t derived_bytes(const Plan& p, size_t elem) {
@@ -294,10 +386,7 @@ ndvm_status run_derive(const Plan& p, const DevPlan& dp, ndvm_dtype dtype, const
     if (di.n_points <= 0) continue;
     const Shape sh = launch_shape(q, elem, di.n_points);
     ReplayArgs a;
-    a.code = dq.code;
-    a.n_code = (int)q.code.size();
-    a.args = dq.args;
-    a.consts = dtype == NDVM_F32 ? (const void*)dq.consts_f : (const void*)dq.consts_d;
+    plan_args(a, q, dq, sh, dtype, err);
     a.obs = obs;
     a.params = static_cast<const char*>(obs) + (size_t)di.base * elem;
     a.loss = nullptr;
@@ -305,12 +394,6 @@ ndvm_status run_derive(const Plan& p, const DevPlan& dp, ndvm_dtype dtype, const
     a.save = static_cast<char*>(ext) + (size_t)(p.n_obs_min + di.offset) * elem;
     a.save_ld = di.n_points;
     a.P = (int)di.stride;
-    a.log2g = sh.log2g;
-    a.shared_lane = sh.shared;
-    a.sstride = sh.sstride;
-    a.staged = sh.staged;
-    a.stage_off = sh.stage_off;
-    a.err = err;
     a.lane0 = 0;
     a.lane_end = di.n_points;
     const int64_t lanes_per_block = sh.tpb >> sh.log2g;
@@ -357,9 +440,9 @@ ndvm_status run(ndvm_tape* t, bool grad, ndvm_dtype dtype, int64_t B, const void
     int64_t fit = (int64_t)(ws_bytes / per_lane);
     if (fit > kMaxChunk) fit = kMaxChunk;
     if (fit < B) {
-      fit -= fit % lanes_per_block;
-      if (fit < lanes_per_block)
-        return fail(NDVM_E_INVALID_ARG, "workspace too small: need at least " + std::to_string(per_lane * lanes_per_block) + " bytes");
+      fit -= fit % sh.chunk_lanes;
+      if (fit < sh.chunk_lanes)
+        return fail(NDVM_E_INVALID_ARG, "workspace too small: need at least " + std::to_string(per_lane * sh.chunk_lanes) + " bytes");
       chunk = fit;
     }
   }
@@ -369,26 +452,13 @@ ndvm_status run(ndvm_tape* t, bool grad, ndvm_dtype dtype, int64_t B, const void
   const DevPlan& dp = grad ? dc->grad : dc->value;
   if (der_bytes > 0 && (s = run_derive(p, dp, dtype, obs, ws, dc->err, stream)) != NDVM_OK) return s;
   ReplayArgs a;
-  // the staged and element-split variants run the paired stream; the plain one does not
-  // carry the paired instruction (it would cost its register budget)
-  const bool paired = (sh.staged || sh.shared) && dp.code_paired != nullptr;
-  a.code = paired ? dp.code_paired : dp.code;
-  a.n_code = (int)(paired ? p.code_paired.size() : p.code.size());
-  a.args = dp.args;
-  a.consts = dtype == NDVM_F32 ? (const void*)dp.consts_f : (const void*)dp.consts_d;
+  plan_args(a, p, dp, sh, dtype, dc->err);
   a.obs = der_bytes > 0 ? ws : obs;  // the extended observations when the tape has shared values
   a.params = params;
   a.loss = loss;
   a.grad = gradp;
   a.save = lane_ws;
   a.save_ld = chunk;
-  a.P = p.n_params;
-  a.log2g = log2g;
-  a.shared_lane = sh.shared;
-  a.sstride = sh.sstride;
-  a.staged = sh.staged;
-  a.stage_off = sh.stage_off;
-  a.err = dc->err;
   for (int64_t l0 = 0; l0 < B; l0 += chunk) {
     a.lane0 = l0;
     a.lane_end = l0 + chunk < B ? l0 + chunk : B;
@@ -409,7 +479,7 @@ ndvm_status run(ndvm_tape* t, bool grad, ndvm_dtype dtype, int64_t B, const void
 // resident blocks per SM of a launch shape (shared memory and registers)
 int resident_blocks(const Shape& s) {
   const int by_smem = (int)(kSmemPerSm / (s.smem + kSmemPerBlockReserved));
-  const int regs = (s.shared || s.staged) ? kMaxRegsStagedOrShared : kMaxRegsPlain;
+  const int regs = (s.shared || s.staged || s.points) ? kMaxRegsStagedOrShared : kMaxRegsPlain;
   const int by_regs = kRegsPerSm / (regs * s.tpb);
   return std::max(1, std::min(by_smem, by_regs));
 }
@@ -427,7 +497,7 @@ struct Member {
 // most kMultiMax members and 2^31 - 1 blocks per launch.
 ndvm_status launch_members(std::vector<Member>& ms, bool f32, void* stream) {
   auto key = [](const Member& m) {
-    return std::vector<int>{m.sh.shared, m.sh.staged, m.sh.log2g, m.sh.tpb, resident_blocks(m.sh)};
+    return std::vector<int>{m.sh.shared, m.sh.staged, m.sh.log2g, m.sh.tpb, resident_blocks(m.sh), m.sh.points};
   };
   std::stable_sort(ms.begin(), ms.end(), [&](const Member& x, const Member& y) { return key(x) < key(y); });
   std::unique_ptr<MultiArgs> table(new MultiArgs);  // about 31 KB: on the heap
@@ -537,10 +607,7 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
         Member m;
         m.sh = launch_shape(dq, elem, di.n_points);
         ReplayArgs& a = m.a;
-        a.code = dd.code;
-        a.n_code = (int)dq.code.size();
-        a.args = dd.args;
-        a.consts = dtype == NDVM_F32 ? (const void*)dd.consts_f : (const void*)dd.consts_d;
+        plan_args(a, dq, dd, m.sh, dtype, dc->err);
         a.obs = obs[k];
         a.params = static_cast<const char*>(obs[k]) + (size_t)di.base * elem;
         a.loss = nullptr;
@@ -548,12 +615,6 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
         a.save = base + (size_t)(p.n_obs_min + di.offset) * elem;
         a.save_ld = di.n_points;
         a.P = (int)di.stride;
-        a.log2g = m.sh.log2g;
-        a.shared_lane = m.sh.shared;
-        a.sstride = m.sh.sstride;
-        a.staged = m.sh.staged;
-        a.stage_off = m.sh.stage_off;
-        a.err = dc->err;
         a.lane0 = 0;
         a.lane_end = di.n_points;
         const int64_t lpb = m.sh.tpb >> m.sh.log2g;
@@ -564,24 +625,13 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
     Member m;
     m.sh = launch_shape(p, elem, B[k]);
     ReplayArgs& a = m.a;
-    const bool paired = (m.sh.staged || m.sh.shared) && dp.code_paired != nullptr;
-    a.code = paired ? dp.code_paired : dp.code;
-    a.n_code = (int)(paired ? p.code_paired.size() : p.code.size());
-    a.args = dp.args;
-    a.consts = dtype == NDVM_F32 ? (const void*)dp.consts_f : (const void*)dp.consts_d;
+    plan_args(a, p, dp, m.sh, dtype, dc->err);
     a.obs = der_bytes > 0 ? (const void*)base : obs[k];
     a.params = params[k];
     a.loss = loss[k];
     a.grad = grad[k];
     a.save = base + der_bytes;
     a.save_ld = B[k];
-    a.P = p.n_params;
-    a.log2g = m.sh.log2g;
-    a.shared_lane = m.sh.shared;
-    a.sstride = m.sh.sstride;
-    a.staged = m.sh.staged;
-    a.stage_off = m.sh.stage_off;
-    a.err = dc->err;
     a.lane0 = 0;
     a.lane_end = B[k];
     const int64_t lpb = m.sh.tpb >> m.sh.log2g;
@@ -633,6 +683,8 @@ ndvm_status ndvm_trace_build(const char* program, size_t len, ndvm_frontend fe, 
     t->tape = std::move(b.t);
     t->grad_plan = make_plan(t->tape, true);
     t->value_plan = make_plan(t->tape, false);
+    compact_plan(t->grad_plan, t->tape.consts);
+    compact_plan(t->value_plan, t->tape.consts);
     std::string why;
     if (!validate_plan(t->grad_plan, t->tape.consts.size(), why) || !validate_plan(t->value_plan, t->tape.consts.size(), why)) {
       delete t;
@@ -864,16 +916,16 @@ ndvm_status ndvm_value_and_grad_noalloc(const ndvm_tape* tape, ndvm_dtype dtype,
                                         " bytes; the fixed scratch holds " + std::to_string(kNoAllocScratchBytes) + " bytes");
   if (p.n_save > 0) {
     const size_t per_lane = (size_t)p.n_save * elem;
-    const size_t per_block = per_lane * lanes_per_block;
+    const size_t per_block = per_lane * sh.chunk_lanes;
     if (per_block > lane_scratch)
       return fail(NDVM_E_INVALID_ARG, "this tape needs " + std::to_string(per_block) + " bytes of workspace per block of " +
-                                          std::to_string(lanes_per_block) + " lanes; the fixed scratch holds " +
+                                          std::to_string(sh.chunk_lanes) + " lanes; the fixed scratch holds " +
                                           std::to_string(kNoAllocScratchBytes) + " bytes");
     int64_t fit = (int64_t)(lane_scratch / per_lane);
-    if (fit < B) chunk = fit - fit % lanes_per_block;
+    if (fit < B) chunk = fit - fit % sh.chunk_lanes;
   }
   // one launch covers at most kMaxChunk lanes, so its grid stays far below 2^31 blocks
-  if (chunk > kMaxChunk) chunk = kMaxChunk - kMaxChunk % lanes_per_block;
+  if (chunk > kMaxChunk) chunk = kMaxChunk - kMaxChunk % sh.chunk_lanes;
   if ((chunk + lanes_per_block - 1) / lanes_per_block > 0x7fffffff)
     return fail(NDVM_E_INVALID_ARG, "too many lanes for one launch");
   DevCache* dc = nullptr;
@@ -896,24 +948,13 @@ ndvm_status ndvm_value_and_grad_noalloc(const ndvm_tape* tape, ndvm_dtype dtype,
     if (s != NDVM_OK) return s;
   }
   ReplayArgs a;
-  const bool paired = (sh.staged || sh.shared) && dc->grad.code_paired != nullptr;
-  a.code = paired ? dc->grad.code_paired : dc->grad.code;
-  a.n_code = (int)(paired ? p.code_paired.size() : p.code.size());
-  a.args = dc->grad.args;
-  a.consts = dtype == NDVM_F32 ? (const void*)dc->grad.consts_f : (const void*)dc->grad.consts_d;
+  plan_args(a, p, dc->grad, sh, dtype, dc->err);
   a.obs = der_bytes > 0 ? scratch : obs;
   a.params = params;
   a.loss = loss;
   a.grad = grad;
   a.save = static_cast<char*>(scratch) + der_bytes;
   a.save_ld = chunk;
-  a.P = p.n_params;
-  a.log2g = log2g;
-  a.shared_lane = sh.shared;
-  a.sstride = sh.sstride;
-  a.staged = sh.staged;
-  a.stage_off = sh.stage_off;
-  a.err = dc->err;
   for (int64_t l0 = 0; l0 < B; l0 += chunk) {
     a.lane0 = l0;
     a.lane_end = l0 + chunk < B ? l0 + chunk : B;

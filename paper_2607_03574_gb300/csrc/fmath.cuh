@@ -49,9 +49,9 @@ __device__ __forceinline__ long long fbits(double x) {
 // The slow paths are calls, not inlined code: a rarely taken branch around inlined library
 // code can be compiled to predicated instructions that issue (all lanes off) every time,
 // and on GB300's FP64 pipe each of those costs a full slot.
-__device__ __noinline__ double slow_exp(double x) { return exp(x); }
-__device__ __noinline__ double slow_log(double x) { return log(x); }
-__device__ __noinline__ double2 slow_sincos(double x) {
+static __device__ __noinline__ double slow_exp(double x) { return exp(x); }
+static __device__ __noinline__ double slow_log(double x) { return log(x); }
+static __device__ __noinline__ double2 slow_sincos(double x) {
   double2 v;
   sincos(x, &v.x, &v.y);
   return v;

@@ -890,6 +890,7 @@ Plan Planner::build_derive(int r, const DeriveInfo& info) const {
     const int xk = load(RK_PARAM, k);
     DInst d;
     d.op = D_FMA;
+    d.flags = kFmaNoGate | kFmaUnitB | kFmaZeroC;
     d.f[0] = mkref(RK_SLOT, next++);
     d.f[1] = mkref(RK_SLOT, xk);
     d.f[2] = mkref(RK_SLOT, one);
@@ -971,7 +972,9 @@ int Planner::const_index(double v) {
 // accumulation rounds once where the general rules round twice.
 void Planner::lower_fma() {
   const PArg one = R(kref(RK_CONST, one_const_));
-  const PArg mzero = R(kref(RK_CONST, const_index(-0.0)));
+  const int mzero_idx = const_index(-0.0);
+  const PArg mzero = R(kref(RK_CONST, mzero_idx));
+  auto is_const = [](const PArg& a, int idx) { return a.isref && a.r.kind == RK_CONST && a.r.id + a.r.off == idx; };
   const int n = (int)code_.size();
   std::vector<PInst> out;
   out.reserve(n + n / 2);
@@ -979,7 +982,8 @@ void Planner::lower_fma() {
   auto fma = [&](PArg dst, PArg a, bool neg, PArg b, PArg c, PArg zs, PArg save) {
     PInst q;
     q.d.op = D_FMA;
-    q.d.flags = neg ? 1 : 0;
+    q.d.flags = (uint8_t)((neg ? 1 : 0) | (is_const(zs, one_const_) ? kFmaNoGate : 0) |
+                          (is_const(b, one_const_) ? kFmaUnitB : 0) | (is_const(c, mzero_idx) ? kFmaZeroC : 0));
     q.f[0] = dst; q.f[1] = a; q.f[2] = b; q.f[3] = c; q.f[4] = zs; q.f[5] = save;
     out.push_back(q);
   };
@@ -996,7 +1000,10 @@ void Planner::lower_fma() {
       case D_SUB: fma(f[0], f[2], true, one, f[1], one, f[3]); break;
       case D_MUL: fma(f[0], f[1], false, f[2], mzero, one, f[3]); break;
       case D_NEG: fma(f[0], f[1], true, one, mzero, one, f[3]); break;
-      case D_ACC: fma(f[0], f[1], false, one, f[0], one, I(-1)); break;
+      case D_ACC:
+        fma(f[0], f[1], false, one, f[0], one, I(-1));
+        out.back().d.flags |= kFmaAcc;
+        break;
       case B_ADD: case B_SUB:
         upd(f[1], fa, f[0], false, one);
         upd(f[2], fb, f[0], p.d.op == B_SUB, one);
@@ -1194,7 +1201,7 @@ void Planner::coalesce_copies() {
   for (int pc = 0; pc < n; pc++) {
     PInst& c = code_[pc];
     if (c.d.op == D_FMA) {
-      if (c.d.flags != 0 || !is_const(c.f[2], one_const_) || !is_const(c.f[3], mzero)) continue;
+      if ((c.d.flags & 1) || !is_const(c.f[2], one_const_) || !is_const(c.f[3], mzero)) continue;
       if (c.f[5].isref || c.f[5].v != -1 || root(vr_of(c.f[4])) != root(vr_of(c.f[1]))) continue;
       if (try_merge(pc, 0, 1, 4)) drop[pc] = 1;
     } else if (c.d.op == B_MADD || c.d.op == B_MSUB) {

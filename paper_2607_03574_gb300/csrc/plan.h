@@ -83,7 +83,8 @@ enum DOp : uint8_t {
                     // observations of the current data point (DOBS refs, inside a data-axis loop)
   // ---- fused multiply-add form of the cheap scalar rules ----
   D_FMA,            // slot f0 = (is_zero(slot f4) ? slot f3 : fma(+-slot f1, slot f2, slot f3)), f5 save;
-                    // flags bit0 negates the first factor.  f4 is the zero-skip test (an adjoint
+                    // flags bit0 negates the first factor (and kFma*: which operands are the stand-ins
+                    // of an absent one).  f4 is the zero-skip test (an adjoint
                     // whose contribution vanishes when it is exactly zero; the slot holding 1.0
                     // when there is none)
   D_FMA2,           // two D_FMA without saves in one record: (f0 dst, f1, f2, f3, f4 zero-skip)
@@ -106,6 +107,10 @@ bool slot_operand(int op, int field);
 constexpr int kFetchPairs = 4;
 constexpr int kFetchStride = 16;
 constexpr int kFetchWindows = 4;
+
+// D_FMA flags: operands that stand in for an absent one (f4 = 1.0, f2 = 1.0, f3 = -0.0), and
+// a data-axis body's accumulation over its points (f0 += f1)
+constexpr uint8_t kFmaNoGate = 2, kFmaUnitB = 4, kFmaZeroC = 8, kFmaAcc = 16;
 
 // "no save" in the 24-bit save fields of D_FMA2
 constexpr int32_t kNoSave24 = 0xFFFFFF;
@@ -136,6 +141,8 @@ struct DeriveInfo {
   double work = 0;                             // DFMA-equivalents per point
 };
 
+constexpr int kCompactWords = 8;
+
 struct Plan {
   bool grad = false;          // has a reverse sweep
   bool spill = false;         // reverse reads primals from the HBM workspace
@@ -150,6 +157,11 @@ struct Plan {
   // the same stream with adjacent independent D_FMA paired into D_FMA2 (for the staged
   // and element-split kernel variants; the plain variant runs `code`)
   std::vector<DInst> code_paired;
+  // the stream's compact records (compact.h), kCompactWords words each, for the scalar
+  // kernels; empty when an instruction has no compact form
+  std::vector<uint32_t> compact;
+  int32_t compact_slots = 0;   // slots of the compact form
+  int64_t compact_points = 0;  // points of its largest data-axis region (0: none)
   std::vector<int32_t> args;
   std::vector<double> extra_consts;  // appended after the tape's constant pool
   // algorithmic cost per lane (for the roofline): DFMA-equivalents and saved bytes

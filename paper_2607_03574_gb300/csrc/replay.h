@@ -10,7 +10,6 @@ namespace ndvm {
 
 struct ReplayArgs {
   const DInst* code;     // device instruction stream
-  int n_code;
   const int32_t* args;   // device operand lists
   const void* consts;    // device constant pool in the compute type
   const void* obs;       // device observations
@@ -18,17 +17,25 @@ struct ReplayArgs {
   void* loss;            // device B losses
   void* grad;            // device B x P gradients (gradient plans only)
   void* save;            // device workspace [element][lane in chunk]
+  int* err;              // device flag set on an invalid instruction
   int64_t lane0;         // first lane of this launch
   int64_t lane_end;      // one past the last lane of this launch
   int64_t save_ld;       // workspace column count (lanes per chunk)
+  int n_code;
   int P;
-  int log2g;             // threads per lane = 1 << log2g
-  int shared_lane;       // 1: the lane's threads share one slot column and split matrix elements
   int sstride;           // slot row stride in elements (threads per block, or lanes per block + pad)
-  int* err;              // device flag set on an invalid instruction
-  int staged;            // 1: the instruction stream is staged through shared memory in chunks
   int stage_off;         // byte offset of the two chunk buffers in dynamic shared memory
+  int16_t log2g;         // threads per lane = 1 << log2g
+  int16_t shared_lane;   // 1: the lane's threads share one slot column and split matrix elements
+  int16_t staged;        // 1: the instruction stream is staged through shared memory in chunks
+  // compact streams (scalar.cu): points per thread and pass, 0 for the general kernels.  code
+  // then holds n_code compact records, staged tells whether they are read in chunks, sstride is
+  // the slots of a thread and stage_off the byte offset of the slot columns.
+  int16_t points;
 };
+
+// Points per thread of a data-axis pass (scalar.cu): one 16-byte access per slot.
+constexpr int kPointsF64 = 2, kPointsF32 = 4;
 
 cudaError_t launch_replay(const ReplayArgs& a, bool f32, int blocks, int tpb, size_t smem, cudaStream_t s);
 
@@ -44,6 +51,10 @@ struct MultiArgs {
 };
 static_assert(sizeof(MultiArgs) <= 32000, "kernel parameter space");
 cudaError_t launch_replay_multi(const MultiArgs& m, bool f32, int blocks, int tpb, size_t smem, cudaStream_t s);
+
+// The kernels of compact streams: one replay (a) or a batch (m).
+cudaError_t launch_scalar(const ReplayArgs* a, const MultiArgs* m, bool f32, int blocks, int tpb, size_t smem,
+                          cudaStream_t s);
 
 // Device-to-device copies of up to kCopyRunsMax runs of 4-byte words in one launch.
 constexpr int kCopyRunsMax = 1000;
