@@ -18,7 +18,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libndvm.so")
 
-SOURCES = ["tape.cpp", "trace_scheme.cpp", "trace_bytecode.cpp", "plan.cpp", "compact.cpp", "capi.cpp", "replay.cu", "scalar.cu"]
+SOURCES = ["tape.cpp", "trace_scheme.cpp", "trace_bytecode.cpp", "plan.cpp", "compact.cpp", "capi.cpp", "replay.cu", "scalar.cu", "matrix.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

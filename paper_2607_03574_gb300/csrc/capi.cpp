@@ -39,6 +39,7 @@ struct DevPlan {
   std::vector<DevPlan> derive;  // derive plans of the shared per-point values
   DInst* code = nullptr;
   DInst* compact = nullptr;      // the compact records, or null
+  DInst* matrix[2] = {nullptr, nullptr};  // the matrix records with their constants in binary64 and binary32
   DInst* code_paired = nullptr;  // the paired stream (staged and element-split variants), or null
   int32_t* args = nullptr;
   double* consts_d = nullptr;
@@ -70,7 +71,7 @@ namespace {
 
 void free_plan(DevPlan& p) {
   for (DevPlan& d : p.derive) free_plan(d);
-  cudaFree(p.code); cudaFree(p.compact); cudaFree(p.code_paired); cudaFree(p.args); cudaFree(p.consts_d); cudaFree(p.consts_f);
+  cudaFree(p.code); cudaFree(p.compact); cudaFree(p.matrix[0]); cudaFree(p.matrix[1]); cudaFree(p.code_paired); cudaFree(p.args); cudaFree(p.consts_d); cudaFree(p.consts_f);
   p = DevPlan{};
 }
 
@@ -100,6 +101,21 @@ ndvm_status upload_plan(const Tape& t, const Plan& p, DevPlan& d) {
     d.compact = static_cast<DInst*>(c);
     if ((e = cudaMemcpy(c, p.compact.data(), sizeof(uint32_t) * p.compact.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
       return cuda_fail(e, "cudaMemcpy");
+  }
+  for (int f32 = 0; f32 < 2 && !p.matrix.empty(); f32++) {
+    // records, constants, lists, each part padded to 16 bytes
+    const size_t rb = sizeof(uint32_t) * p.matrix.size(), cb = (p.matrix_consts.size() * (f32 ? 4 : 8) + 15) / 16 * 16,
+                 lb = (p.matrix_lists.size() * 4 + 15) / 16 * 16;
+    std::vector<char> image(rb + cb + lb);
+    std::memcpy(image.data(), p.matrix.data(), rb);
+    const std::vector<float> f(p.matrix_consts.begin(), p.matrix_consts.end());
+    if (f32) std::copy_n(reinterpret_cast<const char*>(f.data()), f.size() * 4, image.data() + rb);
+    else std::copy_n(reinterpret_cast<const char*>(p.matrix_consts.data()), p.matrix_consts.size() * 8, image.data() + rb);
+    std::copy_n(reinterpret_cast<const char*>(p.matrix_lists.data()), p.matrix_lists.size() * 4, image.data() + rb + cb);
+    void* c = nullptr;
+    if ((e = cudaMalloc(&c, image.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    d.matrix[f32] = static_cast<DInst*>(c);
+    if ((e = cudaMemcpy(c, image.data(), image.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   }
   d.derive.resize(p.derive.size());
   for (size_t k = 0; k < p.derive.size(); k++) {
@@ -339,8 +355,11 @@ void plan_args(ReplayArgs& a, const Plan& p, const DevPlan& d, const Shape& sh, 
   // the staged and element-split variants run the paired stream; the plain one does not
   // carry the paired instruction (it would cost its register budget)
   const bool paired = (sh.staged || sh.shared) && d.code_paired != nullptr;
-  a.code = sh.points ? d.compact : paired ? d.code_paired : d.code;
-  a.n_code = (int)(sh.points ? p.compact.size() / kCompactWords : paired ? p.code_paired.size() : p.code.size());
+  const bool matrix = sh.points && sh.shared;
+  a.n_consts = (int)p.matrix_consts.size();
+  a.n_lists = (int)p.matrix_lists.size();
+  a.code = matrix ? d.matrix[dtype == NDVM_F32] : sh.points ? d.compact : paired ? d.code_paired : d.code;
+  a.n_code = (int)(matrix ? p.matrix.size() / kMatrixWords : sh.points ? p.compact.size() / kCompactWords : paired ? p.code_paired.size() : p.code.size());
   a.args = d.args;
   a.consts = dtype == NDVM_F32 ? (const void*)d.consts_f : (const void*)d.consts_d;
   a.P = p.n_params;
@@ -353,13 +372,36 @@ void plan_args(ReplayArgs& a, const Plan& p, const DevPlan& d, const Shape& sh, 
   a.err = err;
 }
 
+// The launch shape of matrix records: the general kernels' threads per lane and per block, with
+// the records' chunks, the constant matrices and the staged operands' slots in shared memory.
+bool matrix_shape(const Plan& p, size_t elem, const Shape& g, Shape* out) {
+  if (p.matrix.empty() || !g.shared || (1 << g.log2g) > 32) return false;
+  Shape s = g;
+  const size_t fixed = 2 * kMChunk * kMatrixWords * 4 + (p.matrix_consts.size() * elem + 15) / 16 * 16 +
+                       (p.matrix_lists.size() * 4 + 15) / 16 * 16;
+  s.points = 1;
+  s.staged = 1;
+  s.stage_off = (int)fixed;
+  // more threads per lane where that keeps four blocks of 128 on an SM (8-state filters, 16384
+  // lanes x 120 steps: 23.6 ms with 8 threads per lane, 12 warps per SM; 21.4 with 16 and 20)
+  while (s.log2g < 4 && fixed + (size_t)p.matrix_slots * ((s.tpb >> s.log2g) + 1) * elem > kSmemLimit / 4) s.log2g++;
+  for (;; s.tpb /= 2) {  // (the general kernels' block may not leave room for the rest)
+    s.sstride = (s.tpb >> s.log2g) + 1;
+    s.smem = fixed + (size_t)p.matrix_slots * s.sstride * elem;
+    if (s.smem <= kSmemLimit) break;
+    if (s.tpb <= 32 || s.tpb / 2 < (1 << s.log2g)) return false;
+  }
+  *out = s;
+  return true;
+}
+
 // A partial launch (a workspace smaller than all lanes need) covers a multiple of the general
 // kernels' lanes per block, whichever kernel runs: the smallest workspace a call accepts
 // depends on the tape and its lanes only.
 Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
   const Shape g = general_shape(p, elem, B);
   Shape s = g;
-  if (!compact_shape(p, elem, B, &s)) s = g;
+  if (!matrix_shape(p, elem, g, &s) && !compact_shape(p, elem, B, &s)) s = g;
   s.chunk_lanes = g.tpb >> g.log2g;
   return s;
 }

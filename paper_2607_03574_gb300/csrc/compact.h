@@ -47,8 +47,45 @@ enum COp : uint32_t {
   C_GREDUCE,    // w2 slots from w1 on: sums over the thread's points and the lane's threads
   C_LOSS,       // loss = w1
   C_GRAD,       // gradient w2 = w1 (kCNone: 0)
+  // matrices (matrix records, 16 words; matrix.cu).  A matrix operand is a slot or, by the flags,
+  // an index into the stream's constants; w7 workspace of the result as above
+  // products: w1 (rows x cols) = X Y over K terms, element (i, j) = sum over q of X[i xi + q xq]
+  // Y[q yq + j yj]; w2 X, w3 Y, w4 = rows | cols << 8 | K << 16, w5 = xi | xq << 16, w6 = yq | yj << 16,
+  // w9 2^20 / cols rounded up.  Forward (M_F + K, K = 0 for more than 8): w7 save; kMPost: w11 = w12
+  // +- the product too, its save w13 (kMPostNeg, kMPostConst).  Reverse (M_R + K): w10 elements of the
+  // gating operand; kMAcc: added to w1, kCNeg: subtracted; kMGateX, kMGateY: an all-zero X (Y)
+  // contributes nothing
+  M_F, M_F1, M_F2, M_F3, M_F4, M_F5, M_F6, M_F7, M_F8,
+  M_R, M_R1, M_R2, M_R3, M_R4, M_R5, M_R6, M_R7, M_R8,
+  M_FSPARSE,    // the same with one operand constant, by the list at w8: NZ (w4 >> 24) words per element
+  M_RSPARSE,    // of the result, constant's index | other operand's element << 16, kCNone for none
+  M_SELECT,     // elements of a slot run w2 by the list at w8 (kCNone: 0); otherwise as M_F
+  M_RSELECT,    // the same as M_R without kMAcc
+  M_ADD,        // w1 = w2 + w3 (kCNeg: -), w4 elements; slots
+  M_COPY,       // w1 = w2 (kCNeg: -), w4 elements
+  M_ADDC,       // w1 = w2 + w3 (kCNeg: -), w4 elements; slots or constants
+  M_SCALE,      // w1 = w2 (scalar) * w3, w4 elements
+  M_INV,        // w1 = inverse of w2, w3 scratch, w4 n | (2^20 / n rounded up) << 8
+  M_DET, M_LOGDET,  // w1 of w2, w3 and w4 as above, w5 inverse to slots, w6 inverse to workspace
+  M_TRACE,      // w1 of w2, w4 n
+  M_GATHER,     // w1 = elements named by args[w2 ...], w3 of them
+  M_FETCH,      // asynchronous copies of w3 elements from workspace (kMFromObs: observations) w2 on into w1
+  M_RSCALE,     // w2 target scalar, w3 target matrix, w5 scalar, w6 matrix, w4 elements
+  M_RDET,       // w2 target, w4 as above, w5 determinant (kCNone: log-determinant), w6 inverse
+  M_RTRACE,     // w2 target, w4 n
+  M_RGATHER,    // args[w2 ...]: w3 pairs (target, first)
+  M_RSCATTER,   // w2 target of w5 elements, args[w3 ...]: w4 elements
   C_NOPS
 };
+// matrix record flags (bits the scalar records' flags leave free); bits 24 to 26 of w0: 1 + the
+// groups of copies that may stay pending before the next record (0: no wait)
+constexpr uint32_t kMConstX = 1u << 8, kMConstY = 1u << 9, kMAcc = 1u << 10, kMGateX = 1u << 16, kMGateY = 1u << 17,
+                   kMPost = 1u << 18, kMPostNeg = 1u << 19, kMPostConst = 1u << 20, kMFromObs = 1u << 21,
+                   kMOtherY = 1u << 22;  // products with a list: Y is the operand that varies
+constexpr int kMWaitShift = 24;
+constexpr size_t kMChunk = 32;         // records of a chunk
+constexpr size_t kMMaxConsts = 2048;   // constants a stream may hold in shared memory
+constexpr int kMAhead = 3;             // records between a matrix operand's fetch and its use
 constexpr uint32_t kCHasB = 1u << 8, kCHasC = 1u << 9, kCGate = 1u << 10, kCSave = 1u << 11, kCFirstA = 1u << 12,
                    kCFirstB = 1u << 13, kCCommit = 1u << 14, kCWait = 1u << 15, kCNeg = 1u << 31;
 constexpr int kCCountShift = 16;      // 3 bits: copies of a record, a comparison
@@ -64,6 +101,10 @@ struct alignas(16) CRec {
   uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 };
 static_assert(sizeof(CRec) == 4 * kCompactWords, "CRec layout");
+struct alignas(16) MRec {
+  uint32_t w[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+};
+static_assert(sizeof(MRec) == 4 * kMatrixWords, "MRec layout");
 
 // Slots after the plan's own: the validity of a thread's points, and the constants 1 and -0.
 constexpr int kCSlotValid = 0, kCSlotOne = 1, kCSlotMinusZero = 2, kCExtraSlots = 3;
@@ -71,6 +112,7 @@ constexpr int kCSlotValid = 0, kCSlotOne = 1, kCSlotMinusZero = 2, kCExtraSlots 
 // Sets p.compact, p.compact_slots and p.compact_points (and its derive plans') from p.code and
 // the constant pool (the tape's `consts`, then p.extra_consts); p.compact stays empty when the
 // stream has an instruction without a compact form.
+// For a tape with matrices and no data axis, the same for p.matrix*.
 void compact_plan(Plan& p, const std::vector<double>& consts);
 
 }  // namespace ndvm

@@ -141,7 +141,7 @@ struct DeriveInfo {
   double work = 0;                             // DFMA-equivalents per point
 };
 
-constexpr int kCompactWords = 8;
+constexpr int kCompactWords = 8, kMatrixWords = 16;
 
 struct Plan {
   bool grad = false;          // has a reverse sweep
@@ -162,6 +162,12 @@ struct Plan {
   std::vector<uint32_t> compact;
   int32_t compact_slots = 0;   // slots of the compact form
   int64_t compact_points = 0;  // points of its largest data-axis region (0: none)
+  // the same of a tape with matrices and no data axis (matrix.cu): records of kMatrixWords words,
+  // the constant matrices they read, and the lists of their nonzero elements
+  std::vector<uint32_t> matrix;
+  std::vector<double> matrix_consts;
+  std::vector<int32_t> matrix_lists;
+  int32_t matrix_slots = 0;
   std::vector<int32_t> args;
   std::vector<double> extra_consts;  // appended after the tape's constant pool
   // algorithmic cost per lane (for the roofline): DFMA-equivalents and saved bytes

@@ -31,7 +31,10 @@ struct ReplayArgs {
   // compact streams (scalar.cu): points per thread and pass, 0 for the general kernels.  code
   // then holds n_code compact records, staged tells whether they are read in chunks, sstride is
   // the slots of a thread and stage_off the byte offset of the slot columns.
+  // With shared_lane, code holds matrix records (matrix.cu), then n_consts constants and n_lists
+  // list entries, each part padded to 16 bytes.
   int16_t points;
+  int n_consts, n_lists;
 };
 
 // Points per thread of a data-axis pass (scalar.cu): one 16-byte access per slot.
@@ -54,6 +57,10 @@ cudaError_t launch_replay_multi(const MultiArgs& m, bool f32, int blocks, int tp
 
 // The kernels of compact streams: one replay (a) or a batch (m).
 cudaError_t launch_scalar(const ReplayArgs* a, const MultiArgs* m, bool f32, int blocks, int tpb, size_t smem,
+                          cudaStream_t s);
+
+// The kernels of matrix records.
+cudaError_t launch_matrix(const ReplayArgs* a, const MultiArgs* m, bool f32, int blocks, int tpb, size_t smem,
                           cudaStream_t s);
 
 // Device-to-device copies of up to kCopyRunsMax runs of 4-byte words in one launch.

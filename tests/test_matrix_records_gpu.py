@@ -1,0 +1,86 @@
+"""Matrix records (tapes with matrices and no data axis) against the general interpreter.
+
+A tape built with NDVM_COMPACT=0 runs on the general kernels.  Both run the same plan with the
+same sums in the same order, except that a product with a constant matrix leaves out the terms of its
+zeros (which add nothing), so results agree to a few ulp of the lane's largest component (1e-13 here, R10's
+bound is 1e-12).  Non-finite lanes take every term: they keep their class."""
+import numpy as np
+import pytest
+
+import workloads as W
+from conftest import matrix_program, oracle_ref, rel_check
+
+pytestmark = pytest.mark.gpu
+
+
+def _both(ndvm, w, dtype, monkeypatch):
+    import torch
+    fast = ndvm.trace_build(w.program, w.frontend)
+    monkeypatch.setenv("NDVM_COMPACT", "0")
+    general = ndvm.trace_build(w.program, w.frontend)
+    monkeypatch.delenv("NDVM_COMPACT")
+    p = torch.tensor(w.params, dtype=dtype, device="cuda")
+    o = torch.tensor(w.obs, dtype=dtype, device="cuda")
+    out = [ndvm.value_and_grad(t, p, o) + (ndvm.forward(t, p, o),) for t in (fast, general)]
+    torch.cuda.synchronize()
+    for t in (fast, general):
+        ndvm.check_device(t)
+    return [[x.cpu().numpy().astype(np.float64) for x in r] for r in out]
+
+
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+@pytest.mark.parametrize("make", [
+    *[lambda B=B, T=T: W.kalman_cv4(B=B, T=T) for B, T in ((1, 1), (2, 3), (7, 40), (33, 5), (1000, 3), (5000, 2), (20000, 2))],
+    *[lambda n=n, m=m, B=B: W.kalman_rand8(B=B, T=4, n=n, m=m, seed=n)
+      for n, m, B in ((2, 1, 5), (3, 3, 31), (4, 2, 300), (5, 4, 64), (6, 1, 1), (7, 5, 17), (8, 8, 40), (8, 3, 9000), (12, 7, 9),
+                      (16, 6, 20))],
+    *[lambda D=D: W.kalman_highd(B=5, D=D, m=min(D, 8), T=2) for D in (9, 20, 24, 32)],
+    *[lambda k=k: W.Workload("m", matrix_program(np.random.default_rng(1000 + k)), 0,
+                             np.random.default_rng(k).normal(0, 0.5, (3 + 9 * k, 4)), np.zeros(1), np.zeros(4))
+      for k in range(30)]])
+def test_matrix_records_equal_general(ndvm, oracle_mod, cuda, monkeypatch, make, dtype):
+    import torch
+    w = make()
+    fast, general = _both(ndvm, w, getattr(torch, dtype), monkeypatch)
+    if dtype == "float64":
+        ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-13)
+        assert ok, rep
+        idx = np.unique([0, w.B // 2, w.B - 1])
+        ol, og, sp = oracle_ref(oracle_mod, w.program, w.params[idx], w.obs)
+        ok, rep = rel_check(fast[0][idx], fast[1][idx], ol, og, 1e-12, sp)
+        assert ok, rep
+    else:
+        ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-4)
+        assert ok, rep
+    np.testing.assert_array_equal(fast[0], fast[2])
+
+
+SPARSE = ("(define H (matrix 2 3 1.0 0 0 0 0 2.0)) (define S (matrix 3 3 0 1.0 0 1.0 0 0 0 0 1.0))\n"
+          "(model (params a b c) (let* ((X (matrix 3 3 a b 0.5 c a 1.0 b c 2.0)) (Y (matmul S (matmul X S))) (Z (matmul H Y))\n"
+          "   (V (matmul Z (matrix 3 1 a 0.0 b))) (Q (matmul (matmul H X) (transpose H))))\n"
+          "  (+ (mref V 0 0) (mref V 1 0) (trace Q) (mref Z 1 2) (* c (mref Y 0 1)) (trace (matmul X (zeros 3 3))))))")
+
+
+def test_constant_zeros_and_non_finite_values(ndvm, cuda, monkeypatch):
+    """0 * inf is NaN: a warp that has met an infinity or a NaN takes the constants' zero terms."""
+    import torch
+    s = np.array([0.0, -0.0, 1.0, -2.5, np.inf, -np.inf, np.nan, 5e-324, 1e308, -1e200])
+    a, b, c = np.meshgrid(s, s, s)
+    w = W.Workload("sparse", SPARSE, 0, np.stack([a.ravel(), b.ravel(), c.ravel()], 1), np.zeros(1), np.zeros(3))
+    fast, general = _both(ndvm, w, torch.float64, monkeypatch)
+    for f, g in zip(fast, general):
+        np.testing.assert_array_equal(f, g)  # (NaN equals NaN, 0 equals -0)
+
+
+def test_matrix_records_in_chunks(ndvm, cuda, monkeypatch):
+    """A workspace for part of the lanes: the launches over the parts give the same bits."""
+    import torch
+    w = W.kalman_cv4(B=777, T=9)
+    tape = ndvm.trace_build(w.program)
+    p, o = torch.tensor(w.params, device="cuda"), torch.tensor(w.obs, device="cuda")
+    l1, g1 = ndvm.value_and_grad(tape, p, o)
+    per_lane = tape.workspace_bytes(1)
+    l2, g2 = ndvm.value_and_grad(tape, p, o, ws_bytes=per_lane * 130)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(l1.cpu().numpy(), l2.cpu().numpy())
+    np.testing.assert_array_equal(g1.cpu().numpy(), g2.cpu().numpy())
