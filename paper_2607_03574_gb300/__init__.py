@@ -97,9 +97,10 @@ class Tape:
 
     @property
     def handle(self):
-        if not self._h:
+        h = self._h
+        if not h:
             raise NdvmError(1, "tape already freed")
-        return self._h
+        return h
 
     def info(self) -> dict:
         lib = load()
@@ -175,25 +176,33 @@ def measure_op_cost(name: str, iters: int = 2000, stream=None) -> float:
     return v.value
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t) -> int:
     torch = _torch()
-    if t.dtype == torch.float64:
+    dtype = t.dtype
+    if dtype is torch.float64:
         return F64
-    if t.dtype == torch.float32:
+    if dtype is torch.float32:
         return F32
     raise NdvmError(1, f"unsupported dtype {t.dtype}")
 
 
 def _stream_ptr(stream):
+    """The raw handle of `stream` (None: the current stream of the current device)."""
     torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _dev_ptr(t, name):
@@ -203,28 +212,39 @@ def _dev_ptr(t, name):
         raise NdvmError(1, f"{name} must be a CUDA tensor (the replay has no CPU path)")
     if not t.is_contiguous():
         raise NdvmError(1, f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+class _NoContext:
+    def __enter__(self):
+        return None
+
+    def __exit__(self, *exc):
+        return False
+
+
+_current = _NoContext()
 
 
 def _on_stream(stream):
     """Context in which allocations belong to `stream` (the stream the replay runs on):
     torch's caching allocator then reuses a freed block only for later work on that
-    stream, never while a kernel queued there may still use it."""
-    torch = _torch()
-    return torch.cuda.stream(stream if stream is not None else torch.cuda.current_stream())
+    stream, never while a kernel queued there may still use it.  (Without a stream they
+    belong to the current one as it is: entering a stream's context costs more than a
+    small replay's launch.)"""
+    return _current if stream is None else _torch().cuda.stream(stream)
 
 
 def forward(tape: Tape, params, obs, loss=None, stream=None):
     """Per-lane loss.  params: (B, P) CUDA tensor; obs: 1-d CUDA tensor (same dtype).
     An output this call allocates belongs to `stream` (torch's allocator)."""
-    torch = _torch()
     B = params.shape[0]
     if loss is None:
         with _on_stream(stream):
-            loss = torch.empty(B, dtype=params.dtype, device=params.device)
-    _check(load().ndvm_forward(tape.handle, _dtype_code(params), B, _dev_ptr(params, "params"),
-                               _dev_ptr(obs, "obs"), 0 if obs is None else obs.numel(), _dev_ptr(loss, "loss"),
-                               _stream_ptr(stream)))
+            loss = params.new_empty(B)
+    _check((_lib or load()).ndvm_forward(tape.handle, _dtype_code(params), B, _dev_ptr(params, "params"),
+                                         _dev_ptr(obs, "obs"), 0 if obs is None else obs.numel(),
+                                         _dev_ptr(loss, "loss"), _stream_ptr(stream)))
     return loss
 
 
@@ -255,25 +275,27 @@ def value_and_grad(tape: Tape, params, obs, loss=None, grad=None, workspace=None
     """Per-lane loss and gradient.  Returns (loss[B], grad[B, P]).  Outputs and the
     default workspace that this call allocates belong to `stream` (torch's allocator);
     a caller-given workspace must stay allocated until the replay on `stream` is done."""
-    torch = _torch()
+    lib = _lib or load()
     B = params.shape[0]
-    with _on_stream(stream):
-        if loss is None:
-            loss = torch.empty(B, dtype=params.dtype, device=params.device)
-        if grad is None:
-            grad = torch.empty_like(params)
+    if loss is None or grad is None:
+        with _on_stream(stream):
+            if loss is None:
+                loss = params.new_empty(B)
+            if grad is None:
+                grad = _torch().empty_like(params)
     dt = _dtype_code(params)
+    sp = _stream_ptr(stream)
     if workspace is None:
-        need = tape.workspace_bytes(B, dt) if ws_bytes is None else ws_bytes
-        key = (str(params.device), _stream_ptr(stream).value)
-        workspace = _default_ws.setdefault(key, Workspace()).get(need, params.device, stream)
+        need = lib.ndvm_workspace_bytes(tape.handle, B, dt) if ws_bytes is None else ws_bytes
+        if need:
+            key = (str(params.device), sp)
+            workspace = _default_ws.setdefault(key, Workspace()).get(need, params.device, stream)
     nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     if ws_bytes is not None:
         nbytes = min(nbytes, ws_bytes)
-    _check(load().ndvm_value_and_grad(tape.handle, dt, B, _dev_ptr(params, "params"), _dev_ptr(obs, "obs"),
-                                      0 if obs is None else obs.numel(), _dev_ptr(loss, "loss"),
-                                      _dev_ptr(grad, "grad"), _dev_ptr(workspace, "workspace"), nbytes,
-                                      _stream_ptr(stream)))
+    _check(lib.ndvm_value_and_grad(tape.handle, dt, B, _dev_ptr(params, "params"), _dev_ptr(obs, "obs"),
+                                   0 if obs is None else obs.numel(), _dev_ptr(loss, "loss"),
+                                   _dev_ptr(grad, "grad"), _dev_ptr(workspace, "workspace"), nbytes, sp))
     return loss, grad
 
 
@@ -292,27 +314,30 @@ def value_and_grad_multi(tapes, params, obs, loss=None, grad=None, workspace=Non
     for p in params:
         if _dtype_code(p) != dt:
             raise NdvmError(1, "every params tensor must have the same dtype")
-    with _on_stream(stream):
-        if loss is None:
-            loss = [torch.empty(p.shape[0], dtype=p.dtype, device=p.device) for p in params]
-        if grad is None:
-            grad = [torch.empty_like(p) for p in params]
+    lanes = [p.shape[0] for p in params]
+    if loss is None or grad is None:
+        empty_like = torch.empty_like
+        with _on_stream(stream):
+            if loss is None:
+                loss = [p.new_empty(b) for p, b in zip(params, lanes)]
+            if grad is None:
+                grad = [empty_like(p) for p in params]
     Arr = ctypes.c_void_p * n
     I64A = ctypes.c_int64 * n
     th = Arr(*[t.handle for t in tapes])
-    B = I64A(*[p.shape[0] for p in params])
-    lib = load()
+    B = I64A(*lanes)
+    lib = _lib or load()
     need = lib.ndvm_workspace_bytes_multi(th, n, B, dt)
-    if workspace is None:
-        key = (str(params[0].device), _stream_ptr(stream).value, "multi")
+    sp = _stream_ptr(stream)
+    if workspace is None and need:
+        key = (str(params[0].device), sp, "multi")
         workspace = _default_ws.setdefault(key, Workspace()).get(need, params[0].device, stream)
     nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(lib.ndvm_value_and_grad_multi(
-        th, n, dt, B, Arr(*[_dev_ptr(p, "params").value for p in params]),
-        Arr(*[None if o is None else _dev_ptr(o, "obs").value for o in obs]),
+        th, n, dt, B, Arr(*[_dev_ptr(p, "params") for p in params]), Arr(*[_dev_ptr(o, "obs") for o in obs]),
         I64A(*[0 if o is None else o.numel() for o in obs]),
-        Arr(*[_dev_ptr(l, "loss").value for l in loss]), Arr(*[_dev_ptr(g, "grad").value for g in grad]),
-        _dev_ptr(workspace, "workspace"), nbytes, _stream_ptr(stream)))
+        Arr(*[_dev_ptr(l, "loss") for l in loss]), Arr(*[_dev_ptr(g, "grad") for g in grad]),
+        _dev_ptr(workspace, "workspace"), nbytes, sp))
     return loss, grad
 
 

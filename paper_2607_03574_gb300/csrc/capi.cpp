@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -49,11 +50,9 @@ struct DevPlan {
 struct DevCache {
   DevPlan grad, value;
   int* err = nullptr;
-  // buffers for the host-pointer entry point
-  void* h_params = nullptr; size_t h_params_bytes = 0;
-  void* h_obs = nullptr; size_t h_obs_bytes = 0;
-  void* h_loss = nullptr; size_t h_loss_bytes = 0;
-  void* h_grad = nullptr; size_t h_grad_bytes = 0;
+  // buffers for the host-pointer entry point: parameters, observations, losses and gradients in
+  // one, and the workspace
+  void* h_io = nullptr; size_t h_io_bytes = 0;
   void* h_ws = nullptr; size_t h_ws_bytes = 0;
 };
 
@@ -531,6 +530,9 @@ struct Member {
   ReplayArgs a;
   int64_t blocks;
   Shape sh;
+  std::array<int, 6> key;  // what members of one launch have in common
+
+  explicit Member(const Shape& s) : sh(s), key{s.shared, s.staged, s.log2g, s.tpb, resident_blocks(s), s.points} {}
 };
 
 // Launches the members in as few kernels as possible: one per run of members with the
@@ -538,18 +540,15 @@ struct Member {
 // the launch's shared memory, its largest member's, costs no member its occupancy), at
 // most kMultiMax members and 2^31 - 1 blocks per launch.
 ndvm_status launch_members(std::vector<Member>& ms, bool f32, void* stream) {
-  auto key = [](const Member& m) {
-    return std::vector<int>{m.sh.shared, m.sh.staged, m.sh.log2g, m.sh.tpb, resident_blocks(m.sh), m.sh.points};
-  };
-  std::stable_sort(ms.begin(), ms.end(), [&](const Member& x, const Member& y) { return key(x) < key(y); });
+  std::stable_sort(ms.begin(), ms.end(), [](const Member& x, const Member& y) { return x.key < y.key; });
   std::unique_ptr<MultiArgs> table(new MultiArgs);  // about 31 KB: on the heap
   for (size_t i = 0; i < ms.size();) {
     MultiArgs& m = *table;
     m.n = 0;
     int64_t blocks = 0;
     size_t smem = 0;
-    const std::vector<int> k = key(ms[i]);
-    while (i < ms.size() && m.n < kMultiMax && key(ms[i]) == k && blocks + ms[i].blocks <= 0x7fffffff) {
+    const std::array<int, 6> k = ms[i].key;
+    while (i < ms.size() && m.n < kMultiMax && ms[i].key == k && blocks + ms[i].blocks <= 0x7fffffff) {
       m.start[m.n] = (int)blocks;
       m.a[m.n] = ms[i].a;
       blocks += ms[i].blocks;
@@ -600,19 +599,21 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
   if (dtype != NDVM_F64 && dtype != NDVM_F32) return fail(NDVM_E_INVALID_ARG, "bad dtype");
   if (ws && (reinterpret_cast<uintptr_t>(ws) & 255)) return fail(NDVM_E_INVALID_ARG, "workspace must be 256-byte aligned");
   const size_t elem = dtype == NDVM_F32 ? sizeof(float) : sizeof(double);
+  std::vector<Shape> shapes((size_t)n);
   for (int32_t k = 0; k < n; k++) {
-    const std::string at = " (tape " + std::to_string(k) + ")";
-    if (!tapes[k]) return fail(NDVM_E_INVALID_ARG, "null tape" + at);
-    if (B[k] < 0) return fail(NDVM_E_INVALID_ARG, "B must be >= 0" + at);
-    if (B[k] > (int64_t)1 << 40) return fail(NDVM_E_INVALID_ARG, "B too large" + at);
+    auto refuse = [k](ndvm_status s, const char* m) { return fail(s, std::string(m) + " (tape " + std::to_string(k) + ")"); };
+    if (!tapes[k]) return refuse(NDVM_E_INVALID_ARG, "null tape");
+    if (B[k] < 0) return refuse(NDVM_E_INVALID_ARG, "B must be >= 0");
+    if (B[k] > (int64_t)1 << 40) return refuse(NDVM_E_INVALID_ARG, "B too large");
     if (B[k] == 0) continue;
     const Plan& p = tapes[k]->grad_plan;
-    if (p.n_params > 0 && (!params[k] || !grad[k])) return fail(NDVM_E_INVALID_ARG, "null params or grad" + at);
-    if (!loss[k]) return fail(NDVM_E_INVALID_ARG, "null loss" + at);
-    if (n_obs[k] < p.n_obs_min) return fail(NDVM_E_INVALID_ARG, "obs holds too few values" + at);
-    if (p.n_obs_min > 0 && !obs[k]) return fail(NDVM_E_INVALID_ARG, "null obs" + at);
-    if (launch_shape(p, elem, B[k]).smem > kSmemLimit)
-      return fail(NDVM_E_UNSUPPORTED, "tape needs more slots per lane than shared memory holds" + at);
+    if (p.n_params > 0 && (!params[k] || !grad[k])) return refuse(NDVM_E_INVALID_ARG, "null params or grad");
+    if (!loss[k]) return refuse(NDVM_E_INVALID_ARG, "null loss");
+    if (n_obs[k] < p.n_obs_min) return refuse(NDVM_E_INVALID_ARG, "obs holds too few values");
+    if (p.n_obs_min > 0 && !obs[k]) return refuse(NDVM_E_INVALID_ARG, "null obs");
+    shapes[(size_t)k] = launch_shape(p, elem, B[k]);
+    if (shapes[(size_t)k].smem > kSmemLimit)
+      return refuse(NDVM_E_UNSUPPORTED, "tape needs more slots per lane than shared memory holds");
   }
   std::vector<size_t> off;
   const size_t need = multi_layout(tapes, n, B, elem, &off);
@@ -646,8 +647,7 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
         const DeriveInfo& di = p.derive_info[q];
         const DevPlan& dd = dp.derive[q];
         if (di.n_points <= 0) continue;
-        Member m;
-        m.sh = launch_shape(dq, elem, di.n_points);
+        Member m(launch_shape(dq, elem, di.n_points));
         ReplayArgs& a = m.a;
         plan_args(a, dq, dd, m.sh, dtype, dc->err);
         a.obs = obs[k];
@@ -664,8 +664,7 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
         der.push_back(m);
       }
     }
-    Member m;
-    m.sh = launch_shape(p, elem, B[k]);
+    Member m(shapes[(size_t)k]);
     ReplayArgs& a = m.a;
     plan_args(a, p, dp, m.sh, dtype, dc->err);
     a.obs = der_bytes > 0 ? (const void*)base : obs[k];
@@ -792,7 +791,7 @@ void ndvm_tape_free(ndvm_tape* t) {
     DevCache& c = kv.second;
     free_plan(c.grad); free_plan(c.value);
     cudaFree(c.err);
-    cudaFree(c.h_params); cudaFree(c.h_obs); cudaFree(c.h_loss); cudaFree(c.h_grad); cudaFree(c.h_ws);
+    cudaFree(c.h_io); cudaFree(c.h_ws);
   }
   if (!t->dev.empty()) cudaSetDevice(cur);
   delete t;
@@ -827,8 +826,12 @@ ndvm_status ndvm_value_and_grad_multi(const ndvm_tape* const* tapes, int32_t n_t
                                       const void* const* params, const void* const* obs, const int64_t* n_obs,
                                       void* const* loss, void* const* grad, void* workspace, size_t ws_bytes,
                                       void* stream) {
-  return run_multi(const_cast<ndvm_tape* const*>(tapes), n_tapes, dtype, B, params, obs, n_obs, loss, grad, workspace,
-                   ws_bytes, stream);
+  try {
+    return run_multi(const_cast<ndvm_tape* const*>(tapes), n_tapes, dtype, B, params, obs, n_obs, loss, grad, workspace,
+                     ws_bytes, stream);
+  } catch (const std::bad_alloc&) {
+    return fail(NDVM_E_OOM, "host allocation failed");
+  }
 }
 
 }  // extern "C"
@@ -851,22 +854,48 @@ ndvm_status host_replay(const ndvm_tape* tape, ndvm_dtype dtype, int64_t B, cons
   const bool want_grad = grad != nullptr;
   size_t wsb = want_grad ? ndvm_workspace_bytes(t, B, dtype) : 0;
   std::lock_guard<std::mutex> lk(t->host_mu);
-  if ((s = ensure(&dc->h_params, &dc->h_params_bytes, pb)) != NDVM_OK) return s;
-  if ((s = ensure(&dc->h_obs, &dc->h_obs_bytes, ob)) != NDVM_OK) return s;
-  if ((s = ensure(&dc->h_loss, &dc->h_loss_bytes, lb)) != NDVM_OK) return s;
-  if (want_grad && (s = ensure(&dc->h_grad, &dc->h_grad_bytes, pb)) != NDVM_OK) return s;
+  const size_t gb = want_grad ? pb : 0;
+  auto pad = [](size_t n) { return (n + 255) / 256 * 256; };
+  const size_t in = pad(pb) + ob, out = pad(lb) + gb;  // two runs: inputs, then outputs
+  if ((s = ensure(&dc->h_io, &dc->h_io_bytes, pad(in) + out)) != NDVM_OK) return s;
   if (wsb && (s = ensure(&dc->h_ws, &dc->h_ws_bytes, wsb)) != NDVM_OK) return s;
+  char* d_params = static_cast<char*>(dc->h_io);
+  char* d_obs = d_params + pad(pb);
+  char* d_loss = d_params + pad(in);
+  char* d_grad = d_loss + pad(lb);
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
-  if (pb && (e = cudaMemcpyAsync(dc->h_params, params, pb, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(e, "copy params");
-  if (ob && (e = cudaMemcpyAsync(dc->h_obs, obs, ob, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(e, "copy obs");
+  // A synchronous call's small inputs and outputs travel as one copy each way, through a buffer of
+  // this call: a transfer's fixed cost (about 8 us) is more than copying 64 KB on the host
+  constexpr size_t kOneCopy = 64 * 1024;
+  std::vector<char> host;
+  if (sync && pb && ob && in <= kOneCopy) {
+    host.resize(in);
+    std::memcpy(host.data(), params, pb);
+    std::memcpy(host.data() + pad(pb), obs, ob);
+    if ((e = cudaMemcpyAsync(d_params, host.data(), in, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(e, "copy inputs");
+  } else {
+    if (pb && (e = cudaMemcpyAsync(d_params, params, pb, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(e, "copy params");
+    if (ob && (e = cudaMemcpyAsync(d_obs, obs, ob, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(e, "copy obs");
+  }
   if (want_grad)
-    s = run(t, true, dtype, B, dc->h_params, n_obs ? dc->h_obs : nullptr, n_obs, dc->h_loss, dc->h_grad, dc->h_ws, wsb, stream);
+    s = run(t, true, dtype, B, d_params, n_obs ? d_obs : nullptr, n_obs, d_loss, d_grad, dc->h_ws, wsb, stream);
   else
-    s = run(t, false, dtype, B, dc->h_params, n_obs ? dc->h_obs : nullptr, n_obs, dc->h_loss, nullptr, nullptr, 0, stream);
-  if (s != NDVM_OK) return s;
-  if ((e = cudaMemcpyAsync(loss, dc->h_loss, lb, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(e, "copy loss");
-  if (want_grad && pb && (e = cudaMemcpyAsync(grad, dc->h_grad, pb, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(e, "copy grad");
+    s = run(t, false, dtype, B, d_params, n_obs ? d_obs : nullptr, n_obs, d_loss, nullptr, nullptr, 0, stream);
+  if (s != NDVM_OK) {
+    if (!host.empty()) cudaStreamSynchronize(st);  // (the copy may still read this call's buffer)
+    return s;
+  }
+  if (sync && gb && out <= kOneCopy) {
+    std::vector<char> back(out);
+    if ((e = cudaMemcpyAsync(back.data(), d_loss, out, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(e, "copy outputs");
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "synchronize");
+    std::memcpy(loss, back.data(), lb);
+    std::memcpy(grad, back.data() + pad(lb), gb);
+    return NDVM_OK;
+  }
+  if ((e = cudaMemcpyAsync(loss, d_loss, lb, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(e, "copy loss");
+  if (gb && (e = cudaMemcpyAsync(grad, d_grad, gb, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(e, "copy grad");
   if (sync && (e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "synchronize");
   return NDVM_OK;
 }
@@ -877,12 +906,20 @@ extern "C" {
 
 ndvm_status ndvm_value_and_grad_host(const ndvm_tape* tape, ndvm_dtype dtype, int64_t B, const void* params,
                                      const void* obs, int64_t n_obs, void* loss, void* grad, void* stream) {
-  return host_replay(tape, dtype, B, params, obs, n_obs, loss, grad, stream, true);
+  try {
+    return host_replay(tape, dtype, B, params, obs, n_obs, loss, grad, stream, true);
+  } catch (const std::bad_alloc&) {
+    return fail(NDVM_E_OOM, "host allocation failed");
+  }
 }
 
 ndvm_status ndvm_value_and_grad_host_async(const ndvm_tape* tape, ndvm_dtype dtype, int64_t B, const void* params,
                                            const void* obs, int64_t n_obs, void* loss, void* grad, void* stream) {
-  return host_replay(tape, dtype, B, params, obs, n_obs, loss, grad, stream, false);
+  try {
+    return host_replay(tape, dtype, B, params, obs, n_obs, loss, grad, stream, false);
+  } catch (const std::bad_alloc&) {
+    return fail(NDVM_E_OOM, "host allocation failed");
+  }
 }
 
 ndvm_status ndvm_check_device(const ndvm_tape* tape) {
