@@ -412,13 +412,23 @@ size_t derived_bytes(const Plan& p, size_t elem) {
   return ((size_t)(p.n_obs_min + p.derived_elems) * elem + 255) / 256 * 256;
 }
 
-// Fill the extended observations at `ext`: copy obs[0 .. n_obs_min), then run the derive
+// Compact streams read the observations where they are, and the regions' blocks from the extended
+// ones (args, which scalar records do not use, points to them); the general kernels find both there.
+bool reads_both(const Shape& sh) { return sh.points > 0 && !sh.shared; }
+
+void set_obs(ReplayArgs& a, const Shape& sh, const void* obs, const void* ext) {
+  if (ext && reads_both(sh)) a.args = static_cast<const int32_t*>(ext);
+  a.obs = ext && !reads_both(sh) ? ext : obs;
+}
+
+// Fill the extended observations at `ext`: copy obs[0 .. n_obs_min) if `copy`, then run the derive
 // plans, one lane per point of each region, each lane's parameters being its point's
 // observation record (params = obs + base, P = stride).
-ndvm_status run_derive(const Plan& p, const DevPlan& dp, ndvm_dtype dtype, const void* obs, void* ext, int* err,
-                       void* stream) {
+ndvm_status run_derive(const Plan& p, const DevPlan& dp, ndvm_dtype dtype, const void* obs, void* ext, bool copy,
+                       int* err, void* stream) {
   const size_t elem = dtype == NDVM_F32 ? sizeof(float) : sizeof(double);
-  cudaError_t e = cudaMemcpyAsync(ext, obs, (size_t)p.n_obs_min * elem, cudaMemcpyDeviceToDevice, (cudaStream_t)stream);
+  cudaError_t e = cudaSuccess;
+  if (copy) e = cudaMemcpyAsync(ext, obs, (size_t)p.n_obs_min * elem, cudaMemcpyDeviceToDevice, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "copy observations");
   for (size_t k = 0; k < p.derive.size(); k++) {
     const Plan& q = p.derive[k];
@@ -491,10 +501,10 @@ ndvm_status run(ndvm_tape* t, bool grad, ndvm_dtype dtype, int64_t B, const void
   ndvm_status s = device_cache(t, &dc);
   if (s != NDVM_OK) return s;
   const DevPlan& dp = grad ? dc->grad : dc->value;
-  if (der_bytes > 0 && (s = run_derive(p, dp, dtype, obs, ws, dc->err, stream)) != NDVM_OK) return s;
+  if (der_bytes > 0 && (s = run_derive(p, dp, dtype, obs, ws, !reads_both(sh), dc->err, stream)) != NDVM_OK) return s;
   ReplayArgs a;
   plan_args(a, p, dp, sh, dtype, dc->err);
-  a.obs = der_bytes > 0 ? ws : obs;  // the extended observations when the tape has shared values
+  set_obs(a, sh, obs, der_bytes > 0 ? ws : nullptr);
   a.params = params;
   a.loss = loss;
   a.grad = gradp;
@@ -530,17 +540,31 @@ struct Member {
   ReplayArgs a;
   int64_t blocks;
   Shape sh;
-  std::array<int, 6> key;  // what members of one launch have in common
+  std::array<int, 6> key;  // what members of one launch have in common (last: resident blocks per SM)
 
-  explicit Member(const Shape& s) : sh(s), key{s.shared, s.staged, s.log2g, s.tpb, resident_blocks(s), s.points} {}
+  explicit Member(const Shape& s) : sh(s), key{s.shared, s.staged, s.log2g, s.tpb, s.points, resident_blocks(s)} {}
 };
 
 // Launches the members in as few kernels as possible: one per run of members with the
-// same kernel variant, block size, threads per lane and resident blocks per SM (so that
-// the launch's shared memory, its largest member's, costs no member its occupancy), at
-// most kMultiMax members and 2^31 - 1 blocks per launch.
+// same kernel variant, block size and threads per lane.  The launch's shared memory is its largest
+// member's, which may cost the others resident blocks: members of different resident blocks per
+// SM share a launch as long as all of its blocks are on the SMs at once.  (24 programs x 64 lanes:
+// two launches instead of seven, one after the other, of which none filled the chip.)  At most
+// kMultiMax members and 2^31 - 1 blocks per launch.
 ndvm_status launch_members(std::vector<Member>& ms, bool f32, void* stream) {
   std::stable_sort(ms.begin(), ms.end(), [](const Member& x, const Member& y) { return x.key < y.key; });
+  // (within a kind, fewest resident blocks -- most shared memory -- first)
+  for (size_t i = 0; i < ms.size();) {
+    const std::array<int, 6> k = ms[i].key;
+    int64_t blocks = 0;
+    size_t j = i;
+    for (; j < ms.size() && std::equal(k.begin(), k.end() - 1, ms[j].key.begin()); j++) {
+      if (ms[j].key != k && blocks + ms[j].blocks > num_sms() * k.back()) break;
+      blocks += ms[j].blocks;
+    }
+    for (size_t q = i; q < j; q++) ms[q].key = k;
+    i = j;
+  }
   std::unique_ptr<MultiArgs> table(new MultiArgs);  // about 31 KB: on the heap
   for (size_t i = 0; i < ms.size();) {
     MultiArgs& m = *table;
@@ -635,7 +659,7 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
     const size_t der_bytes = derived_bytes(p, elem);
     if (der_bytes > 0) {
       // the observations the program reads, then the derive plans (one lane per point)
-      if (p.n_obs_min > 0) {
+      if (p.n_obs_min > 0 && !reads_both(shapes[(size_t)k])) {
         if (runs->n == kCopyRunsMax) { run_batches.push_back(*runs); runs->n = 0; }
         runs->src[runs->n] = obs[k];
         runs->dst[runs->n] = base;
@@ -667,7 +691,7 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
     Member m(shapes[(size_t)k]);
     ReplayArgs& a = m.a;
     plan_args(a, p, dp, m.sh, dtype, dc->err);
-    a.obs = der_bytes > 0 ? (const void*)base : obs[k];
+    set_obs(a, m.sh, obs[k], der_bytes > 0 ? base : nullptr);
     a.params = params[k];
     a.loss = loss[k];
     a.grad = grad[k];
@@ -1023,12 +1047,12 @@ ndvm_status ndvm_value_and_grad_noalloc(const ndvm_tape* tape, ndvm_dtype dtype,
   cudaError_t e = noalloc_scratch(&scratch);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
   if (der_bytes > 0) {
-    ndvm_status s = run_derive(p, dc->grad, dtype, obs, scratch, dc->err, stream);
+    ndvm_status s = run_derive(p, dc->grad, dtype, obs, scratch, !reads_both(sh), dc->err, stream);
     if (s != NDVM_OK) return s;
   }
   ReplayArgs a;
   plan_args(a, p, dc->grad, sh, dtype, dc->err);
-  a.obs = der_bytes > 0 ? scratch : obs;
+  set_obs(a, sh, obs, der_bytes > 0 ? scratch : nullptr);
   a.params = params;
   a.loss = loss;
   a.grad = grad;

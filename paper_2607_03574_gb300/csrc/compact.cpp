@@ -252,6 +252,8 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
         seed = pending_seed;
         MRec& c = rec(C_LOOP, (uint32_t)f[0], (uint32_t)f[1]);
         c.w[3] = (uint32_t)f[2];
+        for (const DeriveInfo& di : p.derive_info)
+          if (f[1] == 1 && f[2] == p.n_obs_min + di.offset) c.w[0] |= kCExt;
         c.w[5] = valid;
         loop_pc = (int)code.size() - 1;
         *max_points = std::max<int64_t>(*max_points, f[0]);

@@ -36,7 +36,8 @@ enum COp : uint32_t {
   // the interpreter's inner loop ends at these
   C_END,        // end of the stream
   C_CHUNK,      // end of a chunk (the last of each kCChunk records of a long stream)
-  C_LOOP,       // w1 points, w2 stride, w3 base, w4 pc of the matching C_ENDLOOP, w5 validity slot
+  C_LOOP,       // w1 points, w2 stride, w3 base, w4 pc of the matching C_ENDLOOP, w5 validity slot;
+                // kCExt: the points' values are in the extended observations
   C_ENDLOOP,
   C_LOADC,      // w1 = constant: w2, w3 its binary64 bits (low, high), w4 its binary32 bits
   C_LOADP,      // w1 = parameter w2
@@ -87,7 +88,7 @@ constexpr size_t kMChunk = 32;         // records of a chunk
 constexpr size_t kMMaxConsts = 2048;   // constants a stream may hold in shared memory
 constexpr int kMAhead = 3;             // records between a matrix operand's fetch and its use
 constexpr uint32_t kCHasB = 1u << 8, kCHasC = 1u << 9, kCGate = 1u << 10, kCSave = 1u << 11, kCFirstA = 1u << 12,
-                   kCFirstB = 1u << 13, kCCommit = 1u << 14, kCWait = 1u << 15, kCNeg = 1u << 31;
+                   kCFirstB = 1u << 13, kCCommit = 1u << 14, kCWait = 1u << 15, kCExt = 1u << 15, kCNeg = 1u << 31;
 constexpr int kCCountShift = 16;      // 3 bits: copies of a record, a comparison
 constexpr int kCPendingShift = 20;    // 3 bits: groups that may stay pending after a wait
 constexpr uint32_t kCNone = 0xffffffffu;

@@ -30,7 +30,8 @@ struct ReplayArgs {
   int16_t staged;        // 1: the instruction stream is staged through shared memory in chunks
   // compact streams (scalar.cu): points per thread and pass, 0 for the general kernels.  code
   // then holds n_code compact records, staged tells whether they are read in chunks, sstride is
-  // the slots of a thread and stage_off the byte offset of the slot columns.
+  // the slots of a thread, stage_off the byte offset of the slot columns, and args the extended
+  // observations of a tape with shared per-point values.
   // With shared_lane, code holds matrix records (matrix.cu), then n_consts constants and n_lists
   // list entries, each part padded to 16 bytes.
   int16_t points;

@@ -584,6 +584,7 @@ __device__ __forceinline__ void scalar_body(const ReplayArgs& a, const int block
     const int64_t N = r0.y, stride = r0.z, base = r0.w;
     const unsigned end = smem + r1.x * (unsigned)sizeof(CRec), start = rp + (unsigned)sizeof(CRec);
     const uint32_t valid = r1.y;
+    const T* from = (r0.x & kCExt) ? reinterpret_cast<const T*>(a.args) : t.obs;
     const int per = t.G * K;
     for (int64_t p0 = 0; p0 < N; p0 += per) {
       Vec<T, K> on;
@@ -591,7 +592,7 @@ __device__ __forceinline__ void scalar_body(const ReplayArgs& a, const int block
       for (int j = 0; j < K; j++) {
         const int64_t p = p0 + t.grank + (int64_t)j * t.G;
         on.v[j] = p < N ? (T)1 : (T)0;
-        t.point[j] = t.obs + (base + (p < N ? p : N - 1) * stride);
+        t.point[j] = from + (base + (p < N ? p : N - 1) * stride);
       }
       t.template st<K>(valid, on);
       rp = start;
