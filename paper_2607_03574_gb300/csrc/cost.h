@@ -4,12 +4,12 @@
 // zero.  A function counts the FP64 instructions one call executes on GB300, counted
 // by ncu (smsp__inst_executed_pipe_fp64 per call) on the cost probe
 // (ndvm_measure_op_cost: four independent chains per thread on every SM, finite
-// ordinary arguments), less the chain's one add or multiply: the replay's own exp 10
-// and log 13 (fmath.cuh; the same counts in the source, and in ncu counts of
+// ordinary arguments), less the chain's one add or multiply: the replay's own exp 7
+// and log 11 (fmath.cuh; the same counts in the source, and in ncu counts of
 // single-function programs through the replay), and CUDA's tanh 24, sqrt 8, division 8,
 // reciprocal 5, log 29.75 (inside pow's adjoint) and pow 84.  Each call's device time on the probe agrees with its
 // instruction count within 5 %.  The replay's own sin (or cos) and sincos (fmath.cuh)
-// execute 16 and 19 FP64 instructions (counted in the source; the probe's device time
+// execute 14 and 17 FP64 instructions (counted in the source; the probe's device time
 // per call, 16.7 and 19.5 DFMA with the chain's add, agrees).  The roofline divides
 // this work by the FP64 pipe's peak issue rate.
 #pragma once
@@ -18,14 +18,14 @@
 namespace ndvm {
 namespace cost {
 
-constexpr double kExp = 10, kLog = 13, kSin = 16, kSinCos = 19, kTanh = 24, kSqrt = 8,
+constexpr double kExp = 7, kLog = 11, kSin = 14, kSinCos = 17, kTanh = 24, kSqrt = 8,
                  kRcp = 5, kPow = 84, kDiv = 8, kLogLib = 29.75;
-// A division in a data-axis body takes 1/b from the hardware estimate and two Newton
-// steps (kRcpNewton: four fused multiply-adds) and one correction step (a product and
+// A division in a data-axis body takes 1/b from the hardware estimate and one third-order
+// step (kRcpNewton: three fused multiply-adds) and one correction step (a product and
 // two fused multiply-adds, kDivStep); its reverse rule divides the adjoint by b with the
 // forward sweep's reciprocal (kDivStep).  A lane-level division is the IEEE division
 // (kDiv) in both sweeps.  The log's adjoint divides the same way as a body division.
-constexpr double kDivStep = 3, kRcpNewton = 4;
+constexpr double kDivStep = 3, kRcpNewton = 3;
 
 // (the reciprocal of a determinant or pivot is the correctly rounded rcp)
 inline double inv_cost(int n) {

@@ -1,21 +1,22 @@
 // Double-precision exp and log for the replay kernel, written for GB300's FP64
 // pipe: a warp's FP64 instruction occupies its scheduler's share of the FP64 unit for
-// 64 cycles (2 fused multiply-adds per clock per SM), so range reduction, table indexing,
+// 64 cycles (2 fused multiply-adds per clock per SM), so table indexing,
 // exponent scaling and the special-case tests run on the integer pipes and the
 // FP64 pipe does only the arithmetic that needs 53-bit precision.
 //
 // exp: table-driven method of P. T. P. Tang (ACM TOMS 15(2), 1989).  x = (64m + j)
 //   ln2/64 + r with |r| <= ln2/128; exp(x) = 2^m 2^(j/64) (1 + p(r)), p the Taylor
 //   polynomial of exp(r) - 1 through r^5 (truncation < 4e-17 relative).  The
-//   nearest integer 64m + j comes from adding 1.5 * 2^52 (no conversion
-//   instruction); 2^m is applied by an integer add to the exponent field.
-//   10 FP64 instructions.
+//   nearest integer 64m + j comes from binary32 arithmetic, as does the polynomial's r^4
+//   coefficient; 2^m is applied by an integer add to the exponent field.
+//   7 FP64 instructions (10 with both in binary64, at the same error).
 // log: table-driven method of P. T. P. Tang (ACM TOMS 16(4), 1990).  x = 2^e m with
 //   m in [0.75, 1.5), F = j/128 the nearest table point, f = m - F (exact),
 //   u = f / F by a tabulated reciprocal, log x = e ln2 + ln F + log1p(u) with the
 //   Taylor polynomial of log1p through u^7 (|u| <= 1/192; truncation < 2e-17
 //   relative).  For m near 1, F = 1 and the result is log1p(u) alone, so there is
-//   no cancellation.  13 FP64 instructions.
+//   no cancellation.  11 FP64 instructions (e is converted by integer operations, and the last
+//   coefficient computed in binary32; 13 without, at the same error).
 // sin, cos: additive range reduction of W. J. Cody and W. Waite ("Software Manual for
 //   the Elementary Functions", 1980) by pi/64: x = n pi/64 + r, |r| <= pi/128, with pi/64
 //   in three parts (n times the first two exact for |n| < 2^20), then the addition
@@ -23,11 +24,14 @@
 //   sin x = S + (S (cos r - 1) + C sin r), cos x = C + (C (cos r - 1) - S sin r),
 //   S = sin(k pi/64), C = cos(k pi/64), with sin r through r^7 and cos r - 1 through r^6
 //   (truncation below 4e-19 relative at |r| = pi/128).  No branch on the quadrant: every
-//   lane of a warp runs the same instructions.  16 FP64 instructions for one of them, 19
-//   for both.
+//   lane of a warp runs the same instructions.  14 FP64 instructions for one of them, 17
+//   for both (n by binary32 arithmetic; 16 and 19 without).
 // Arguments outside the fast range (|x| >= 708 for exp; x <= 0, subnormal, infinite
 // or NaN for log; |x| >= 2^15, infinite or NaN for sin and cos) take CUDA's functions.
-// Results are within about 1 ulp (sin and cos: 2 ulp, tested).
+// Results are within about 1 ulp (sin and cos: 2 ulp, tested).  Against 64-bit mantissas over a
+// million arguments a range, error with the binary32 parts and without them: exp on +-1 1.245
+// ulp at most, rms 0.4104 (1.255, 0.4108); on +-707 1.249, 0.4113 (1.249, 0.4117); log on [0.7, 1.6]
+// 1.519, 0.4363 both ways; sin on +-1000 1.768, 0.3941 both ways.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -57,16 +61,35 @@ static __device__ __noinline__ double2 slow_sincos(double x) {
   return v;
 }
 
+// double to float and back by integer operations, off the FP64 pipe (a conversion instruction
+// may take a slot there).  to_f32 truncates, and gives 0 below float's normal range; finite
+// arguments below 2^127 only.  to_f64 is exact for zeros and normal numbers.
+__device__ __forceinline__ float to_f32(double x) {
+  const unsigned hi = (unsigned)((unsigned long long)fbits(x) >> 32), lo = (unsigned)fbits(x), m = hi & 0x7fffffffu;
+  unsigned s = __funnelshift_l(lo, m, 3) - (896u << 23);
+  if (m < 0x38100000u) s = 0;
+  return __uint_as_float(s | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = m ? ((m >> 3) + 0x38000000u) | (b & 0x80000000u) : 0u;
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// the integer nearest to x * scale (within 2^-20 of a tie either one), in binary32
+__device__ __forceinline__ float nearest(double x, float scale) { return fmaf(to_f32(x), scale, 12582912.0f); }
+__device__ __forceinline__ int nearest_int(float t) { return (int)__float_as_uint(t) - 0x4b400000; }
+__device__ __forceinline__ double nearest_f64(float t) { return to_f64(t - 12582912.0f); }
+
 __device__ __forceinline__ double fast_exp(double x) {
   const long long bx = fbits(x);
   if ((bx & 0x7fffffffffffffffLL) >= 0x4086200000000000LL) return slow_exp(x);  // |x| >= 708, inf, nan
-  const double magic = 0x1.8p52;
-  const double t = fma(x, NDVM_64_LN2, magic);
-  const int n = __double2loint(t);  // nearest integer to 64 x / ln2
-  const double kd = t - magic;
+  const float t = nearest(x, (float)NDVM_64_LN2);
+  const int n = nearest_int(t);  // 64 x / ln2
+  const double kd = nearest_f64(t);
   double r = fma(kd, -NDVM_LN2_64_HI, x);
   r = fma(kd, -NDVM_LN2_64_LO, r);
-  double p = fma(r, NDVM_INV120, NDVM_INV24);
+  double p = to_f64(fmaf(to_f32(r), (float)NDVM_INV120, (float)NDVM_INV24));  // of r^4 (below 4e-11 of the result)
   p = fma(r, p, NDVM_INV6);
   p = fma(r, p, 0.5);
   p = fma(r, p, 1.0);
@@ -93,13 +116,13 @@ __device__ __forceinline__ double fast_log(double x) {
   const double m = __longlong_as_double(mb);
   const double f = m - kLogFv[ix];  // exact
   const double u = f * kLogInvF[ix];
-  double t = fma(u, NDVM_INV7, -NDVM_INV6);
+  double t = to_f64(fmaf(to_f32(u), (float)NDVM_INV7, -(float)NDVM_INV6));  // of u^6 (below 4e-12 of u)
   t = fma(u, t, NDVM_INV5);
   t = fma(u, t, -0.25);
   t = fma(u, t, NDVM_INV3);
   t = fma(u, t, -0.5);
   const double p = fma(u * u, t, u);  // log1p(u)
-  const double ed = __longlong_as_double(0x4338000000000000LL + e) - 0x1.8p52;  // (double)e, exact
+  const double ed = to_f64((float)e);  // exact
   const double hi = fma(ed, NDVM_LN2_HI, kLogF[ix]);
   const double lo = fma(ed, NDVM_LN2_LO, p);
   return hi + lo;
@@ -114,10 +137,9 @@ __device__ __forceinline__ void fast_sincos(double x, double* s, double* c) {
     *c = v.y;
     return;
   }
-  const double magic = 0x1.8p52;
-  const double t = fma(x, NDVM_64_PI, magic);
-  const int n = __double2loint(t);  // nearest integer to 64 x / pi
-  const double kd = t - magic;
+  const float t = nearest(x, (float)NDVM_64_PI);
+  const int n = nearest_int(t);  // 64 x / pi
+  const double kd = nearest_f64(t);
   double r = fma(kd, -NDVM_PI_64_1, x);
   r = fma(kd, -NDVM_PI_64_2, r);
   r = fma(kd, -NDVM_PI_64_3, r);

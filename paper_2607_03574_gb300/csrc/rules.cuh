@@ -86,17 +86,15 @@ template <typename T> __device__ __noinline__ T slow_div(T a, T b) { return a / 
 template <typename T> __device__ __noinline__ T slow_rcp(T b) { return rcp_rn(b); }
 
 // 1/b for b with an exponent within +-500 (div_step_ok): the hardware estimate
-// (rcp.approx.ftz.f64, off the FP64 pipe) refined by two Newton-Raphson steps
-// y <- y + y (1 - b y), each doubling its correct bits; 4 FP64 instructions and no
-// special-case code.  The result is within a hair of half an ulp, which is what the
+// (rcp.approx.ftz.f64, off the FP64 pipe, more than 20 correct bits) refined by one third-order
+// step, y + y (e + e^2) with e = 1 - b y, which triples them; 3 FP64 instructions (two
+// Newton steps take 4) and no special-case code.  The result is within a hair of half an ulp, which is what the
 // correction step of a division needs.
 __device__ __forceinline__ double rcp_newton(double b) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  double e = fma(-b, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-b, y, 1.0);
-  return fma(y, e, y);
+  const double e = fma(-b, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ float rcp_newton(float b) { return __frcp_rn(b); }
 
