@@ -138,6 +138,7 @@ __device__ __forceinline__ T dot_long(unsigned x, unsigned xs, unsigned y, unsig
 
 template <typename T>
 __device__ __noinline__ bool all_zero_at(unsigned a, unsigned s, int n) {
+#pragma unroll 1
   for (int e = 0; e < n; e++)
     if (!is_zero(ld1<T>(a + (unsigned)e * s))) return false;
   return true;
@@ -146,16 +147,15 @@ __device__ __noinline__ bool all_zero_at(unsigned a, unsigned s, int n) {
 // The words of the frequent records as the kernel reads them: once per block and chunk, decode()
 // turns slots and element strides into byte offsets and strides (an operand's offset is from the
 // lane's column, or, for a constant, an address).
-//   w1 result, w2 X, w3 Y, w4 elements / G | elements mod G << 16; and for products: w5 xi, w6 xq,
+//   w1 result, w2 X, w3 Y, w4 elements; and for products: w5 xi, w6 xq,
 //   w7 save, w8 2^20 / cols, w9 yq, w10 yj, w11 and w12 result and operand of the sum that follows,
 //   w13 its save, w14 elements of the gating operand | NZ << 13 | cols << 20, w15 list address | K << 24
 template <typename T>
 __device__ void decode(const ReplayArgs& a, unsigned rp, unsigned consts, unsigned lists) {
   const uint4 r0 = ld_words(rp), r1 = ld_words(rp + 16), r2 = ld_words(rp + 32), r3 = ld_words(rp + 48);
-  const unsigned row = (unsigned)a.sstride * (unsigned)sizeof(T), size = (unsigned)sizeof(T), G = 1u << a.log2g;
+  const unsigned row = (unsigned)a.sstride * (unsigned)sizeof(T), size = (unsigned)sizeof(T);
   auto off = [&](uint32_t slot) { return slot == kCNone ? kCNone : slot / kCSlotUnit * row; };
   auto operand = [&](uint32_t v, bool c) { return c ? consts + v * size : off(v); };
-  auto split = [&](uint32_t n) { return n / G | (n % G) << 16; };
   auto put = [&](unsigned at, uint4 v) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
   };
@@ -168,13 +168,12 @@ __device__ void decode(const ReplayArgs& a, unsigned rp, unsigned consts, unsign
     const unsigned xs = cx ? size : row, ys = cy ? size : row;
     const unsigned rows = r1.x & 0xff, cols = (r1.x >> 8) & 0xff, K = (r1.x >> 16) & 0xff, NZ = r1.x >> 24;
     put(rp, make_uint4(f, off(r0.y), operand(r0.z, cx), operand(r0.w, cy)));
-    put(rp + 16, make_uint4(split(rows * cols), (r1.y & 0xffff) * xs, (r1.y >> 16) * xs, r1.w));
+    put(rp + 16, make_uint4(rows * cols, (r1.y & 0xffff) * xs, (r1.y >> 16) * xs, r1.w));
     put(rp + 32, make_uint4(r2.y, (r1.z & 0xffff) * ys, (r1.z >> 16) * ys, off(r2.w)));
     put(rp + 48, make_uint4((f & kMPost) ? operand(r3.x, f & kMPostConst) : 0u, r3.y, r2.z | NZ << 13 | cols << 20,
                             (lists + 4u * r2.x) | K << 24));
   } else if (op == M_ADD || op == M_COPY) {
     put(rp, make_uint4(f, off(r0.y), off(r0.z), off(r0.w)));
-    put(rp + 16, make_uint4(split(r1.x), r1.y, r1.z, r1.w));
   } else if (op == M_FETCH) {
     put(rp, make_uint4(f, off(r0.y), r0.z, r0.w));
   }
@@ -228,21 +227,22 @@ struct Product {
   }
 };
 
-// The thread's elements of n (w4 of a decoded record): every thread of the warp makes the same
-// passes; one without an element in the last pass repeats the result's last element and does
-// not store it (on = false).
+// The thread's elements of n: every thread of the warp makes the same passes; one without an
+// element in the last pass repeats the result's last element and does not store it (on = false).
+// (One copy of the body, not unrolled: the interpreter's code is larger than the instruction
+// cache, and two copies or unrolled loops cost the 8-state filter 10 %.)
 template <typename T, typename F>
-__device__ __forceinline__ void each_element(const MThread<T>& t, uint32_t w4, F f) {
-  const int full = (int)(w4 & 0xffffu), rem = (int)(w4 >> 16);
+__device__ __forceinline__ void each_element(const MThread<T>& t, int n, F f) {
   int e = t.g;
   unsigned o = (unsigned)t.g * t.row;
-  for (int k = 0; k < full; k++, e += t.G, o += t.step) f(e, o, true);
-  if (rem) {
-    const int last = full * t.G + rem - 1;
-    const bool on = e <= last;
-    e = on ? e : last;
-    f(e, (unsigned)e * t.row, on);
-  }
+#pragma unroll 1
+  do {
+    const bool on = e < n;
+    const int c = on ? e : n - 1;
+    f(c, on ? o : (unsigned)c * t.row, on);
+    e += t.G;
+    o += t.step;
+  } while (e - t.g < n);
 }
 
 // The thread's elements of a product over K terms (K = 0: more than 8).
@@ -251,7 +251,7 @@ __device__ __forceinline__ void dense(const MThread<T>& t, unsigned rp, const ui
   const Product<T, REV> p(t, rp, r0, r1);
   const int cols = p.cols();
   const unsigned X = p.r0.z + ((p.f & kMConstX) ? 0u : t.base), Y = p.r0.w + ((p.f & kMConstY) ? 0u : t.base);
-  each_element(t, r1.x, [&](int e, unsigned o, bool on) {
+  each_element(t, (int)r1.x, [&](int e, unsigned o, bool on) {
     const int i = (int)(((uint32_t)e * p.r2.x) >> 20), j = e - i * cols;
     const unsigned x = X + (unsigned)i * p.r1.y, y = Y + (unsigned)j * p.r2.z;
     const T s = p.start(o);
@@ -269,7 +269,7 @@ __device__ __noinline__ unsigned dense_call(MThread<T> t, unsigned rp, uint4 r0,
   const Product<T, REV> p(t, rp, r0, r1);
   const unsigned X = p.r0.z + ((p.f & kMConstX) ? 0u : t.base), Y = p.r0.w + ((p.f & kMConstY) ? 0u : t.base);
   const int K = (int)(p.r3.w >> 24);
-  each_element(t, r1.x, [&](int e, unsigned o, bool on) {
+  each_element(t, (int)r1.x, [&](int e, unsigned o, bool on) {
     const int i = (int)(((uint32_t)e * p.r2.x) >> 20), j = e - i * p.cols();
     unsigned x = X + (unsigned)i * p.r1.y, y = Y + (unsigned)j * p.r2.z;
     const T s = p.start(o);
@@ -298,10 +298,11 @@ __device__ __forceinline__ void sparse(const MThread<T>& t, unsigned rp, const u
   const uint32_t v = (p.f & kMOtherY) ? r0.w : r0.z;
   const bool both = (p.f & kMConstX) && (p.f & kMConstY);
   const unsigned other = both ? v : t.base + v, step = both ? (unsigned)sizeof(T) : t.row;
-  each_element(t, r1.x, [&](int e, unsigned o, bool on) {
+  each_element(t, (int)r1.x, [&](int e, unsigned o, bool on) {
     const unsigned l = (p.r3.w & 0xffffffu) + 4u * (unsigned)(e * NZ);
     const T s = p.start(o);
     T z = s;
+#pragma unroll 1
     for (int u = 0; u < NZ; u++) {
       const uint32_t q = ld_word(l + 4u * (unsigned)u);
       if (q == kCNone) break;
@@ -317,7 +318,7 @@ template <typename T, bool REV>
 __device__ __forceinline__ void select(const MThread<T>& t, unsigned rp, const uint4& r0, const uint4& r1, Largest& bad) {
   const Product<T, REV> p(t, rp, r0, r1);
   const unsigned other = t.base + ((p.f & kMOtherY) ? r0.w : r0.z), list = p.r3.w & 0xffffffu;
-  each_element(t, r1.x, [&](int e, unsigned o, bool on) {
+  each_element(t, (int)r1.x, [&](int e, unsigned o, bool on) {
     const uint32_t q = ld_word(list + 4u * (unsigned)e);
     T z = ld1<T>(other + (q == kCNone ? 0u : q) * t.row);
     if (q == kCNone) z = (T)0;
@@ -329,7 +330,7 @@ __device__ __forceinline__ void select(const MThread<T>& t, unsigned rp, const u
 template <typename T, bool COPY>
 __device__ __forceinline__ void add(const MThread<T>& t, const uint4& r0, const uint4& r1, Largest& bad) {
   const unsigned out = t.base + r0.y, a = t.base + r0.z, b = t.base + r0.w;
-  each_element(t, r1.x, [&](int e, unsigned o, bool on) {
+  each_element(t, (int)r1.x, [&](int e, unsigned o, bool on) {
     T z;
     if (COPY) z = with_sign(ld1<T>(a + o), r0.x);
     else z = ld1<T>(a + o) + with_sign(ld1<T>(b + o), r0.x);
@@ -431,6 +432,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
     case M_ADDC: {
       const MOperand<T> A(t, r0.z, f & kMConstX), B(t, r0.w, f & kMConstY);
       const unsigned out = t.at(r0.y);
+#pragma unroll 1
       for (int e = t.g; e < (int)r1.x; e += t.G) {
         const T z = A[e] + with_sign(B[e], f);
         bad.see(z);
@@ -443,6 +445,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
       const T s = MOperand<T>(t, r0.z, f & kMConstX)[0];
       const MOperand<T> A(t, r0.w, f & kMConstY);
       const unsigned out = t.at(r0.y);
+#pragma unroll 1
       for (int e = t.g; e < (int)r1.x; e += t.G) {
         const T z = s * A[e];
         bad.see(z);
@@ -462,6 +465,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
     }
     case M_GATHER: {
       const unsigned out = t.at(r0.y);
+#pragma unroll 1
       for (int e = t.g; e < (int)r0.w; e += t.G) {
         const T z = element<T>(t, a, a.args[r0.z + (unsigned)e]);
         bad.see(z);
@@ -472,6 +476,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
     }
     case M_FETCH: {  // (a thread copies the elements that it stored)
       const unsigned out = t.base + r0.y;
+#pragma unroll 1
       for (int e = t.g; e < (int)r0.w; e += t.G) {
         const T* src = (f & kMFromObs) ? t.obs + (r0.z + (unsigned)e) : t.saved(r0.z + (unsigned)e);
         if (sizeof(T) == 8)
@@ -503,7 +508,8 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
           if (fb) zero_own(t, o, w);
         } else {
           const T s = MOperand<T>(t, r1.y, f & kMConstX)[0];
-          for (int e = t.g; e < w; e += t.G) {
+    #pragma unroll 1
+      for (int e = t.g; e < w; e += t.G) {
             const unsigned q = o + (unsigned)e * t.row;
             const T z = fma(s, ld1<T>(g + (unsigned)e * t.row), fb ? neg_zero<T>() : ld1<T>(q));
             bad.see(z);
@@ -524,6 +530,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
       const T fac = r1.y != kCNone ? g * t.template ld<1>(r1.y).v[0] : g;
       const MOperand<T> I(t, r1.z, false);
       const uint32_t mn = r1.x >> 8;
+#pragma unroll 1
       for (int e = t.g; e < n * n; e += t.G) {
         const int i = (int)(((uint32_t)e * mn) >> 20), j = e - i * n;
         const unsigned q = o + (unsigned)e * t.row;
