@@ -373,23 +373,85 @@ void plan_args(ReplayArgs& a, const Plan& p, const DevPlan& d, const Shape& sh, 
 
 // The launch shape of matrix records: the general kernels' threads per lane and per block, with
 // the records' chunks, the constant matrices and the staged operands' slots in shared memory.
-bool matrix_shape(const Plan& p, size_t elem, const Shape& g, Shape* out) {
-  if (p.matrix.empty() || !g.shared || (1 << g.log2g) > 32) return false;
+bool matrix_shape(const Plan& p, size_t elem, int64_t B, const Shape& g, Shape* out) {
+  if (p.matrix.empty() || !g.shared) return false;
   Shape s = g;
   const size_t fixed = 2 * kMChunk * kMatrixWords * 4 + (p.matrix_consts.size() * elem + 15) / 16 * 16 +
                        (p.matrix_lists.size() * 4 + 15) / 16 * 16;
   s.points = 1;
   s.staged = 1;
   s.stage_off = (int)fixed;
+  const size_t lane_bytes = (size_t)p.matrix_slots * elem;
+  const bool alone = s.log2g > 5;  // the general kernel gives a lane a block: its slots fill one
+  if (alone) s.log2g = 4;
   // more threads per lane where that keeps four blocks of 128 on an SM (8-state filters, 16384
   // lanes x 120 steps: 23.6 ms with 8 threads per lane, 12 warps per SM; 21.4 with 16 and 20)
-  while (s.log2g < 4 && fixed + (size_t)p.matrix_slots * ((s.tpb >> s.log2g) + 1) * elem > kSmemLimit / 4) s.log2g++;
-  for (;; s.tpb /= 2) {  // (the general kernels' block may not leave room for the rest)
-    s.sstride = (s.tpb >> s.log2g) + 1;
-    s.smem = fixed + (size_t)p.matrix_slots * s.sstride * elem;
-    if (s.smem <= kSmemLimit) break;
-    if (s.tpb <= 32 || s.tpb / 2 < (1 << s.log2g)) return false;
+  while (s.log2g < 4 && fixed + lane_bytes * (size_t)((s.tpb >> s.log2g) + 1) > kSmemLimit / 4) s.log2g++;
+  // few lanes: more threads while the launch is under a warp per scheduler and each thread has
+  // two elements of the largest matrix (four once a lane spans warps, whose barriers cost more)
+  if (!threads_per_lane_override())
+    while (s.log2g < 8 && (B << s.log2g) < num_sms() * 128 && ((s.log2g < 5 ? 4 : 8) << s.log2g) <= p.matrix_width) s.log2g++;
+  // matrices of 256 elements and more: a lane alone in its block, without the padding of shared
+  // rows, and threads enough for eight warps on an SM (16 states, 2000 lanes x 8 steps: 1.98 ms
+  // with 16 threads per lane in 128-thread blocks, one of which fills an SM)
+  if (alone || ((size_t)p.matrix_width * elem >= 2048 && !threads_per_lane_override())) s.log2g = std::max(s.log2g, 6);
+  if (s.log2g > 5) {  // one lane per block
+    s.smem = fixed + lane_bytes;
+    if (s.smem > kSmemLimit) return false;
+    const int64_t lanes = kSmemPerSm / (s.smem + kSmemPerBlockReserved);
+    while (s.log2g < 8 && lanes << s.log2g < 256 && (4 << s.log2g) <= p.matrix_width) s.log2g++;
+    s.tpb = 1 << s.log2g;
+    s.sstride = 1;
+    // the general kernel's lanes are smaller (no copies of constants): where it also has a block
+    // for each and takes fewer rounds of them, it is faster (48 states in f32, 400 lanes x 4
+    // steps: one round of 1.23 ms against three, 1.64 ms)
+    const int64_t fit = std::min<int64_t>(kSmemPerSm / (g.smem + kSmemPerBlockReserved), kRegsPerSm / (kMaxRegsStagedOrShared * g.tpb));
+    const int64_t here = std::min<int64_t>(lanes, kRegsPerSm / (kMaxRegsStagedOrShared * s.tpb)), sms = num_sms();
+    if (alone && (B + fit * sms - 1) / (fit * sms) < (B + here * sms - 1) / (here * sms)) return false;
+    *out = s;
+    return true;
   }
+  // threads per block: the general kernels', or fewer where an SM then holds more of them, or
+  // more where that saves a round of blocks (9000 lanes x 10 steps of 6 states: blocks of 32 are
+  // two rounds, of 128 one)
+  const int64_t sms = num_sms();
+  auto per_sm = [](const Shape& x) {
+    return (int)std::min<int64_t>(kSmemPerSm / (x.smem + kSmemPerBlockReserved), kRegsPerSm / (kMaxRegsStagedOrShared * x.tpb));
+  };
+  auto rounds = [&](const Shape& x) {
+    const int64_t lanes = (int64_t)per_sm(x) * (x.tpb >> x.log2g) * sms;
+    return (B + lanes - 1) / lanes;
+  };
+  auto blocks_of = [&](int t) {
+    Shape x = s;
+    x.tpb = t;
+    x.sstride = (t >> s.log2g) + 1;
+    x.smem = fixed + lane_bytes * (size_t)x.sstride;
+    return x;
+  };
+  const int most = std::min(std::max(g.tpb, 1 << s.log2g), 128);
+  int best = 0;
+  for (int t = most; t >= 32 && t >= 1 << s.log2g; t /= 2) {
+    const Shape x = blocks_of(t);
+    if (x.smem > kSmemLimit || per_sm(x) * t <= best) continue;
+    best = per_sm(x) * t;
+    s = x;
+  }
+  if (best == 0) return false;
+  const int64_t general = rounds(g);
+  for (int t = 2 * most; t <= 128 && rounds(s) > general; t *= 2) {
+    const Shape x = blocks_of(t);
+    if (x.smem <= kSmemLimit && rounds(x) < rounds(s)) s = x;
+  }
+  // The general kernel where the lanes' larger slot files (their copies of constants) add more
+  // rounds than the records save: from 12 states in f64 half as many again (8000 lanes x 6 steps
+  // of 12 states, five rounds against three: 2.34 ms, 2.18 by the general kernel; 4000 lanes x 10
+  // steps, two against two: 1.75 and 2.58; 15 states, 9000 lanes x 6 steps, five against four:
+  // 3.43 and 4.00), else twice as many of one, or of two with as many threads per lane (4000
+  // lanes x 6 steps of 11 states, two against one: 1.09 ms and 0.89; 16384 lanes x 120 steps of
+  // 8 states, four rounds with 16 threads per lane against two with 8: 19.3 ms and 23.6).
+  if (elem == 8 && p.matrix_width >= 128 && 2 * rounds(s) >= 3 * general) return false;
+  if (s.log2g >= 3 && rounds(s) >= 2 * general && (general == 1 || (general == 2 && s.log2g == g.log2g))) return false;
   *out = s;
   return true;
 }
@@ -400,7 +462,7 @@ bool matrix_shape(const Plan& p, size_t elem, const Shape& g, Shape* out) {
 Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
   const Shape g = general_shape(p, elem, B);
   Shape s = g;
-  if (!matrix_shape(p, elem, g, &s) && !compact_shape(p, elem, B, &s)) s = g;
+  if (!matrix_shape(p, elem, B, g, &s) && !compact_shape(p, elem, B, &s)) s = g;
   s.chunk_lanes = g.tpb >> g.log2g;
   return s;
 }

@@ -864,12 +864,16 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
   p.compact_points = 0;
   if (!compact_enabled()) return;
   if (p.has_matrix) {
-    // (a lane whose slots alone fill the shared memory runs in a block of its own, on the general kernel)
-    if (p.has_regions || (size_t)p.n_slots * 3 * sizeof(float) > (size_t)227 * 1024) return;
+    // (where a lane's slots leave no room for the constants, the general kernel runs)
+    if (p.has_regions || (size_t)p.n_slots * sizeof(double) > (size_t)150 * 1024) return;
     Matrices mx;
     int64_t points = 0;
     std::vector<MRec> code = translate(p, consts, &points, &mx);
     if (code.empty() || mx.consts.size() > kMMaxConsts) return;
+    p.matrix_width = 0;
+    for (const MRec& c : code)
+      if ((c.w[0] & 0xff) >= M_F && (c.w[0] & 0xff) <= M_RSELECT)
+        p.matrix_width = std::max(p.matrix_width, (int32_t)((c.w[4] & 0xff) * ((c.w[4] >> 8) & 0xff)));
     p.matrix_slots = place_stages(code, mx, p.n_slots + kCExtraSlots + 1);
     mark_chunks<MRec, kMChunk>(code);
     for (const MRec& c : code) p.matrix.insert(p.matrix.end(), c.w, c.w + kMatrixWords);

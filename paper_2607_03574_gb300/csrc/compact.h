@@ -85,7 +85,7 @@ constexpr uint32_t kMConstX = 1u << 8, kMConstY = 1u << 9, kMAcc = 1u << 10, kMG
                    kMOtherY = 1u << 22;  // products with a list: Y is the operand that varies
 constexpr int kMWaitShift = 24;
 constexpr size_t kMChunk = 32;         // records of a chunk
-constexpr size_t kMMaxConsts = 2048;   // constants a stream may hold in shared memory
+constexpr size_t kMMaxConsts = 8192;   // constants a stream may hold in shared memory
 constexpr int kMAhead = 3;             // records between a matrix operand's fetch and its use
 constexpr uint32_t kCHasB = 1u << 8, kCHasC = 1u << 9, kCGate = 1u << 10, kCSave = 1u << 11, kCFirstA = 1u << 12,
                    kCFirstB = 1u << 13, kCCommit = 1u << 14, kCWait = 1u << 15, kCExt = 1u << 15, kCNeg = 1u << 31;

@@ -1,7 +1,7 @@
 // Replay of tapes with matrices: an interpreter of matrix records (compact.h), for tapes without
-// a data axis whose lanes share a warp.
+// a data axis.
 //
-// G consecutive threads serve one lane and share its column of slots; they split the elements
+// G consecutive threads of a warp (or block) serve one lane and share its column of slots; they split the elements
 // of each matrix result (element e belongs to thread e mod G) and repeat its scalar records.
 // What bounds these tapes is the latency of a record where lanes are few (a 4 x 4 product is
 // one or two elements per thread: four dependent multiply-adds of 64 cycles, in an interpreter
@@ -20,13 +20,21 @@
 //  - a record's operation word is read from one thread, so that the compiler knows it to be the
 //    same in all of them and leaves out the reconvergence around every test of it (a scalar
 //    record: 88 -> 75 instructions).
+//  - each element loop exists once and is not unrolled: copies per size did not fit in the
+//    instruction cache next to each other (the constant-velocity filter below 5.94 -> 5.62).
+//  - where a lane's slots leave few warps on an SM, or there are few lanes, a lane has a block of
+//    64 to 256 threads (BLOCK), with a barrier of the block after each record.
 // Measured on one GB300 against the general kernel (ms): a 4-state constant-velocity filter of 200
-// steps, 8192 lanes 7.00 -> 5.94 (FP64 instructions halved), 3001 lanes without gradient 2.78 ->
-// 2.08; 256 lanes x 80 steps 2.15 -> 1.85; an 8-state filter of 120 steps, 16384 lanes 23.6 ->
-// 21.5.  What binds now is still instructions: about 118 per record, 6 cycles each with one warp
-// per scheduler.  Tried and not faster: two elements' chains interleaved (cv4 7.1), a thread's
-// elements in one column with its operand in registers (no change), predicated accesses in place
-// of branches.
+// steps, 8192 lanes 6.99 -> 5.62 (FP64 instructions halved), 3001 lanes without gradient 2.78 ->
+// 1.96; 256 lanes x 80 steps 2.15 -> 1.75; an 8-state filter of 120 steps, 16384 lanes 23.6 ->
+// 19.3; a lane per block: 16 states, 50 lanes x 8 steps 1.24 -> 0.48 and 2000 lanes 1.58 -> 1.34;
+// 24 states, 400 lanes x 6 steps 2.12 -> 0.73; 32 states, 1500 lanes x 4 steps 14.2 -> 3.72.
+// What binds now is still instructions: about 118 per record, 6 cycles each with one warp
+// per scheduler.  Tried and not faster: two elements' chains interleaved (the first filter 7.1), a
+// thread's elements in one column with its operand in registers (no change), predicated accesses
+// in place of branches, a warp per lane for 12 to 15 states (the same elements, fewer lanes: 12
+// states, 8000 lanes x 6 steps 2.83 for 2.34), scaled constant matrices read from global memory
+// to save their shared memory (32 states 9 % slower).
 #include "interp.cuh"
 #include "smallmat.cuh"
 
@@ -374,7 +382,7 @@ __device__ __noinline__ unsigned small_matrix(MThread<T> t, unsigned smem0, uint
   L.sbase = reinterpret_cast<T*>(smem_raw + (t.base - smem0));
   L.ss = (int)(t.row / sizeof(T));
   L.eg = t.g;
-  L.es = t.G;
+  L.es = min(t.G, 32);  // (a lane over several warps: the first one)
   const Opnd<T> A = {L.wp((int)(r0.z / kCSlotUnit)), L.ss};
   const int scratch = (int)(r0.w / kCSlotUnit);
   const bool inverse = op == M_INV || r1.y != kCNone || (int)r1.z >= 0;
@@ -396,7 +404,7 @@ __device__ __noinline__ unsigned small_matrix(MThread<T> t, unsigned smem0, uint
   if (inverse) {
     const uint32_t out = op == M_INV ? r0.y : r1.y;
     const int sv = op == M_INV ? ((r0.x & kCSave) ? (int)r1.w : -1) : (int)r1.z;
-    for (int e = t.g; e < n * n; e += t.G) {
+    for (int e = t.g; e < n * n; e += L.es) {
       const T v = n <= 3 ? inv_small(A, n, e, r) : gj_inverse<T>(L, scratch, n, perm, (int)(((uint32_t)e * mn) >> 20), e - (int)(((uint32_t)e * mn) >> 20) * n);
       bad.see(v);
       if (out != kCNone) st1<T>(t.at(out) + (unsigned)e * t.row, v);
@@ -425,7 +433,8 @@ __device__ __forceinline__ void zero_own(const MThread<T>& t, unsigned at, int n
 
 // The matrix records besides products and small inverses.
 template <typename T>
-__device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0, const uint4& r1, const ReplayArgs& a, Largest& bad) {
+__device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0, const uint4& r1, const ReplayArgs& a,
+                                            bool finite, Largest& bad) {
   const uint32_t f = r0.x;
   const bool fa = f & kCFirstA, fb = f & kCFirstB;
   switch (f & 0xff) {
@@ -497,8 +506,15 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
         if (zero) {
           if (fa) s.v[0] = (T)0;
         } else {
+          // (a constant's zeros add nothing to a finite sum; a lane over several warps: the first one)
           const MOperand<T> A(t, r1.z, f & kMConstY);
-          for (int e = 0; e < w; e++) s.v[0] = fma(ld1<T>(g + (unsigned)e * t.row), A[e], s.v[0]);
+          const bool skip = finite && (f & kMConstY);
+          if (t.g < 32)
+#pragma unroll 1
+            for (int e = 0; e < w; e++) {
+              const T x = A[e];
+              if (!skip || !is_zero(x)) s.v[0] = fma(ld1<T>(g + (unsigned)e * t.row), x, s.v[0]);
+            }
         }
         t.template st<1>(r0.z, s);
       }
@@ -595,7 +611,9 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
 template <typename T>
 __device__ __noinline__ void scalar_rule(MThread<T> t, uint4 r0, uint4 r1) { rule<T, 1>(t, r0, r1); }
 
-template <typename T>
+// BLOCK: a lane has the whole block, G = 64 to 256 threads (large matrices, few lanes): a block
+// barrier after every record, scalar records and small inverses in the first warp.
+template <typename T, bool BLOCK>
 __device__ __forceinline__ void matrix_body(const ReplayArgs& a, const int block) {
   const int tid = threadIdx.x, tpb = blockDim.x;
   const unsigned smem = (unsigned)__cvta_generic_to_shared(smem_raw);
@@ -633,8 +651,11 @@ __device__ __forceinline__ void matrix_body(const ReplayArgs& a, const int block
   copy(code + 4 * (int64_t)a.n_code, t.consts, (int)((const_bytes + list_bytes) / 16));
   stage(0, smem);
   Largest bad;
-  // whether a thread of the warp has stored an infinity or a NaN
-  auto met = [&]() { return __any_sync(0xffffffffu, bad.w >= kInfWord<T>); };
+  // whether a thread of the warp (or block) has stored an infinity or a NaN
+  auto met = [&]() -> bool {
+    if (BLOCK) return __syncthreads_or(bad.w >= kInfWord<T>);
+    return __any_sync(0xffffffffu, bad.w >= kInfWord<T>);
+  };
   for (int first = kChunkRecs, k = 0;; first += kChunkRecs, k++) {
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");  // chunk k has landed (and every staged operand)
     __syncthreads();  // for every thread; and every warp has left chunk k - 1: its buffer is free
@@ -653,7 +674,9 @@ __device__ __forceinline__ void matrix_body(const ReplayArgs& a, const int block
 #define NDVM_DENSE(K)                                                      \
   case M_F + K: dense<T, K, false>(t, rp, r0, r1, bad); break;            \
   case M_R + K: dense<T, K, true>(t, rp, r0, r1, bad); break;
-      switch (op) {
+      const bool others = BLOCK && tid >= 32 && ((op < M_F && op != C_FETCH && op != C_CHUNK && op != C_END) ||
+                                                 (op >= M_INV && op <= M_TRACE));
+      if (!others) switch (op) {  // (else the first warp's record)
         case C_ARITH: arith_decoded<T>(t, r0, r1); break;
         NDVM_DENSE(0) NDVM_DENSE(1) NDVM_DENSE(2) NDVM_DENSE(3) NDVM_DENSE(4) NDVM_DENSE(5) NDVM_DENSE(6)
         NDVM_DENSE(7) NDVM_DENSE(8)
@@ -680,7 +703,7 @@ __device__ __forceinline__ void matrix_body(const ReplayArgs& a, const int block
         case C_CHUNK: goto next_chunk;
         case C_END: return;
         default:
-          if (op > M_F) matrix_rule<T>(t, r0, r1, a, bad);
+          if (op > M_F) matrix_rule<T>(t, r0, r1, a, op == M_RSCALE && !met(), bad);
           else if (op < C_END) scalar_rule<T>(t, r0, r1);
           else outer<T, 1, 1>(t, r0, r1, a);
       }
@@ -690,19 +713,21 @@ __device__ __forceinline__ void matrix_body(const ReplayArgs& a, const int block
         if (wait == 1) asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         else asm volatile("cp.async.wait_group 1;\n" ::: "memory");
       }
-      __syncwarp();  // the lane's threads see each other's elements
+      // the lane's threads see each other's elements
+      if (BLOCK) __syncthreads();
+      else __syncwarp();
     }
   next_chunk:;
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128, 4) k_matrix(ReplayArgs a) {
-  matrix_body<T>(a, blockIdx.x);
+template <typename T, bool BLOCK>
+__global__ void __launch_bounds__(BLOCK ? 256 : 128, BLOCK ? 2 : 4) k_matrix(ReplayArgs a) {
+  matrix_body<T, BLOCK>(a, blockIdx.x);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128, 4) k_matrix_multi(const __grid_constant__ MultiArgs ma) {
+template <typename T, bool BLOCK>
+__global__ void __launch_bounds__(BLOCK ? 256 : 128, BLOCK ? 2 : 4) k_matrix_multi(const __grid_constant__ MultiArgs ma) {
   const int b = blockIdx.x;
   int lo = 0, hi = ma.n - 1;
   while (lo < hi) {
@@ -710,24 +735,30 @@ __global__ void __launch_bounds__(128, 4) k_matrix_multi(const __grid_constant__
     if (ma.start[mid] <= b) lo = mid;
     else hi = mid - 1;
   }
-  matrix_body<T>(ma.a[lo], b - ma.start[lo]);
+  matrix_body<T, BLOCK>(ma.a[lo], b - ma.start[lo]);
+}
+
+template <typename T, bool BLOCK>
+cudaError_t launch(const ReplayArgs* a, const MultiArgs* m, int blocks, int tpb, size_t smem, cudaStream_t s) {
+  static SmemLimit one, many;
+  cudaError_t e = m ? many.allow(k_matrix_multi<T, BLOCK>, smem) : one.allow(k_matrix<T, BLOCK>, smem);
+  if (e != cudaSuccess) return e;
+  if (m) k_matrix_multi<T, BLOCK><<<blocks, tpb, smem, s>>>(*m);
+  else k_matrix<T, BLOCK><<<blocks, tpb, smem, s>>>(*a);
+  return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch(const ReplayArgs* a, const MultiArgs* m, int blocks, int tpb, size_t smem, cudaStream_t s) {
-  static SmemLimit one, many;
-  cudaError_t e = m ? many.allow(k_matrix_multi<T>, smem) : one.allow(k_matrix<T>, smem);
-  if (e != cudaSuccess) return e;
-  if (m) k_matrix_multi<T><<<blocks, tpb, smem, s>>>(*m);
-  else k_matrix<T><<<blocks, tpb, smem, s>>>(*a);
-  return cudaGetLastError();
+cudaError_t launch_type(const ReplayArgs* a, const MultiArgs* m, int blocks, int tpb, size_t smem, cudaStream_t s) {
+  return (m ? m->a[0] : *a).log2g > 5 ? launch<T, true>(a, m, blocks, tpb, smem, s)
+                                      : launch<T, false>(a, m, blocks, tpb, smem, s);
 }
 
 }  // namespace
 
 cudaError_t launch_matrix(const ReplayArgs* a, const MultiArgs* m, bool f32, int blocks, int tpb, size_t smem,
                           cudaStream_t s) {
-  return f32 ? launch<float>(a, m, blocks, tpb, smem, s) : launch<double>(a, m, blocks, tpb, smem, s);
+  return f32 ? launch_type<float>(a, m, blocks, tpb, smem, s) : launch_type<double>(a, m, blocks, tpb, smem, s);
 }
 
 }  // namespace ndvm

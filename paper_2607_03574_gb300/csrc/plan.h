@@ -168,6 +168,7 @@ struct Plan {
   std::vector<double> matrix_consts;
   std::vector<int32_t> matrix_lists;
   int32_t matrix_slots = 0;
+  int32_t matrix_width = 0;  // elements of its largest matrix
   std::vector<int32_t> args;
   std::vector<double> extra_consts;  // appended after the tape's constant pool
   // algorithmic cost per lane (for the roofline): DFMA-equivalents and saved bytes

@@ -2,7 +2,7 @@
 
 A tape built with NDVM_COMPACT=0 runs on the general kernels.  Both run the same plan; they
 differ in the order in which a data sum's points are added (points per thread) and in
-roundings of the reverse rules that the compact form fuses, so lanes agree within R10's bound
+roundings of the reverse rules that the compact form fuses, so lanes agree within the parity bound
 (1e-12 in binary64, 1e-5 in binary32, of the lane's largest component).  Sizes cover the edges of the split:
 fewer points than threads, one more or less than a pass, one lane, ragged warps."""
 import numpy as np

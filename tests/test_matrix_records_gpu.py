@@ -2,8 +2,8 @@
 
 A tape built with NDVM_COMPACT=0 runs on the general kernels.  Both run the same plan with the
 same sums in the same order, except that a product with a constant matrix leaves out the terms of its
-zeros (which add nothing), so results agree to a few ulp of the lane's largest component (1e-13 here, R10's
-bound is 1e-12).  Non-finite lanes take every term: they keep their class."""
+zeros (which add nothing), so results agree to a few ulp of the lane's largest component (1e-13 here, the
+parity bound is 1e-12).  Non-finite lanes take every term: they keep their class."""
 import numpy as np
 import pytest
 
@@ -34,7 +34,8 @@ def _both(ndvm, w, dtype, monkeypatch):
     *[lambda n=n, m=m, B=B: W.kalman_rand8(B=B, T=4, n=n, m=m, seed=n)
       for n, m, B in ((2, 1, 5), (3, 3, 31), (4, 2, 300), (5, 4, 64), (6, 1, 1), (7, 5, 17), (8, 8, 40), (8, 3, 9000), (12, 7, 9),
                       (16, 6, 20))],
-    *[lambda D=D: W.kalman_highd(B=5, D=D, m=min(D, 8), T=2) for D in (9, 20, 24, 32)],
+    *[lambda D=D, B=B: W.kalman_highd(B=B, D=D, m=min(D, 8), T=2)
+      for D, B in ((9, 5), (16, 3), (20, 5), (24, 1), (24, 300), (32, 5), (32, 700), (40, 2), (48, 3))],
     *[lambda k=k: W.Workload("m", matrix_program(np.random.default_rng(1000 + k)), 0,
                              np.random.default_rng(k).normal(0, 0.5, (3 + 9 * k, 4)), np.zeros(1), np.zeros(4))
       for k in range(30)]])
