@@ -410,37 +410,47 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
                 if (!(side ? cy : cx) || ref_kind(side ? X : Y) == RK_OBS) continue;
                 const int32_t at = ref_index(side ? Y : X);
                 const int outer = side ? cols : rows, so = side ? yj : xi, sq = side ? yq : xq;
-                bool finite = true, unit = true;
+                bool finite = true, unit = true, odd = false;
                 int most = 1;
                 for (int o = 0; o < outer; o++) {
                   int m = 0;
                   for (int q = 0; q < K; q++) {
                     const double v = pool_at(at, o * so + q * sq);
                     finite = finite && std::isfinite(v);
-                    if (v != 0) { m++; unit = unit && v == 1.0; }
+                    if (v != 0) { m++; unit = unit && v == 1.0; odd = odd || q % 2 == 1; }
                   }
                   most = std::max(most, m);
                 }
                 if (!finite || most >= best) continue;
-                best = nz = most;
+                best = most;
                 const bool select = most == 1 && unit && !(more & kMAcc) && !(side ? cx : cy);
+                // (sums over more than 8 terms take the even and the odd ones in two chains, as the
+                // dense products do: the same roundings whichever kernel a lane runs on)
+                const bool chains = K > 8 && odd && !select;
+                nz = most + (chains ? 1 : 0);
                 std::vector<int32_t> l;
                 for (int i = 0; i < rows; i++)
                   for (int j = 0; j < cols; j++) {
-                    int m = 0;
+                    const size_t end = l.size() + (size_t)nz;
                     const int o = side ? j : i;
-                    for (int q = 0; q < K; q++) {
-                      if (pool_at(at, o * so + q * sq) == 0) continue;
-                      const uint32_t ce = (uint32_t)((side ? y : x) + (uint32_t)(o * so + q * sq));
-                      const uint32_t oe = (uint32_t)(side ? i * xi + q * xq : q * yq + j * yj);
-                      l.push_back((int32_t)(select ? oe : ce | oe << 16));
-                      m++;
+                    auto terms = [&](int from, int step) {
+                      for (int q = from; q < K; q += step) {
+                        if (pool_at(at, o * so + q * sq) == 0) continue;
+                        const uint32_t ce = (uint32_t)((side ? y : x) + (uint32_t)(o * so + q * sq));
+                        const uint32_t oe = (uint32_t)(side ? i * xi + q * xq : q * yq + j * yj);
+                        l.push_back((int32_t)(select ? oe : ce | oe << 16));
+                      }
+                    };
+                    terms(0, chains ? 2 : 1);
+                    if (chains) {
+                      l.push_back((int32_t)kMSplit);
+                      terms(1, 2);
                     }
-                    for (; m < most; m++) l.push_back((int32_t)kCNone);
+                    l.resize(end, (int32_t)kCNone);
                   }
                 list = mx->list(l);
                 op = reverse ? (select ? M_RSELECT : M_RSPARSE) : select ? M_SELECT : M_FSPARSE;
-                flags = (flags & ~kMOtherY) | (side ? 0 : kMOtherY);
+                flags = (flags & ~(kMOtherY | kMChains)) | (side ? 0 : kMOtherY) | (chains ? kMChains : 0);
               }
               // (a variable operand's slots differ from step to step: the list names its elements only)
               products[key] = {op, nz, list, flags & ~had};

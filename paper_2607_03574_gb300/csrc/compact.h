@@ -1,12 +1,13 @@
-// Compact records of scalar and data-axis streams, run by the kernels of scalar.cu.
+// Compact records: scalar and data-axis streams' (32 bytes, run by scalar.cu) and, of twice the
+// size, those of streams with matrices and no data axis (matrix.cu).
 //
 // A Plan's stream (DInst, 48 bytes, operands as kind and index) describes every tape.  A
 // stream made of scalar instructions only is translated once, on the host, into records
 // the interpreter can execute with few instructions of its own: operands are byte offsets
 // into the thread's slot column (one shift-add per operand), constants are part of the
 // record, and the cheap rules share one record kind whose unused operands are not loaded.
-// A record spends about 25 instructions around its arithmetic where the general
-// interpreter spends about 100.
+// A scalar record executes 36 instructions where the general interpreter executes 102, a
+// matrix record 118 for 172 (a logistic recurrence and a 4-state Kalman filter).
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -59,7 +60,7 @@ enum COp : uint32_t {
   M_F, M_F1, M_F2, M_F3, M_F4, M_F5, M_F6, M_F7, M_F8,
   M_R, M_R1, M_R2, M_R3, M_R4, M_R5, M_R6, M_R7, M_R8,
   M_FSPARSE,    // the same with one operand constant, by the list at w8: NZ (w4 >> 24) words per element
-  M_RSPARSE,    // of the result, constant's index | other operand's element << 16, kCNone for none
+  M_RSPARSE,    // of the result, constant's index | other operand's element << 16, kMSplit, kCNone for none
   M_SELECT,     // elements of a slot run w2 by the list at w8 (kCNone: 0); otherwise as M_F
   M_RSELECT,    // the same as M_R without kMAcc
   M_ADD,        // w1 = w2 + w3 (kCNeg: -), w4 elements; slots
@@ -83,6 +84,8 @@ enum COp : uint32_t {
 constexpr uint32_t kMConstX = 1u << 8, kMConstY = 1u << 9, kMAcc = 1u << 10, kMGateX = 1u << 16, kMGateY = 1u << 17,
                    kMPost = 1u << 18, kMPostNeg = 1u << 19, kMPostConst = 1u << 20, kMFromObs = 1u << 21,
                    kMOtherY = 1u << 22;  // products with a list: Y is the operand that varies
+constexpr uint32_t kMChains = 1u << 23;  // products with a list: two chains, by kMSplit
+constexpr uint32_t kMSplit = 0xfffffffeu;  // in a list: the terms of the second chain follow
 constexpr int kMWaitShift = 24;
 constexpr size_t kMChunk = 32;         // records of a chunk
 constexpr size_t kMMaxConsts = 8192;   // constants a stream may hold in shared memory

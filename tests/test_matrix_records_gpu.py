@@ -85,3 +85,24 @@ def test_matrix_records_in_chunks(ndvm, cuda, monkeypatch):
     torch.cuda.synchronize()
     np.testing.assert_array_equal(l1.cpu().numpy(), l2.cpu().numpy())
     np.testing.assert_array_equal(g1.cpu().numpy(), g2.cpu().numpy())
+
+
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+@pytest.mark.parametrize("n,band", [(8, 3), (9, 1), (9, 2), (12, 3), (15, 4), (16, 5), (24, 2)])
+def test_banded_constants_sum_as_dense(ndvm, cuda, monkeypatch, n, band, dtype):
+    # products with a banded constant keep the dense sums' chains: a lane's bits do not depend on the
+    # number of lanes, which chooses the kernel
+    import torch
+    rng = np.random.default_rng(n * 10 + band)
+    F = np.where(np.abs(np.subtract.outer(np.arange(n), np.arange(n))) < band, rng.normal(0, 0.4, (n, n)), 0.0)
+    lit = " ".join(repr(float(v)) if v else "0" for v in F.ravel())
+    eye = " ".join("1.0" if i == j else "0" for i in range(n) for j in range(n))
+    ones = " ".join(repr(float(v)) for v in rng.normal(0, 1, n))
+    text = (f"(define F (matrix {n} {n} {lit})) (define I (matrix {n} {n} {eye})) (define v (matrix {n} 1 {ones}))\n"
+            f"(model (params a b) (let* ((P (m+ (mscale a F) (mscale b I)))"
+            f" (Q (matmul F (matmul P (transpose F)))) (R (matmul Q F)) (s (matmul (transpose v) (matmul R v))))"
+            f" (+ (trace Q) (mref s 0 0))))")
+    w = W.Workload("banded", text, 0, rng.normal(0.5, 0.5, (700, 2)), np.zeros(1), np.zeros(2))
+    fast, general = _both(ndvm, w, getattr(torch, dtype), monkeypatch)
+    for x, y in zip(fast, general):
+        np.testing.assert_array_equal(x, y)
