@@ -9,8 +9,7 @@
 // single-function programs through the replay), and CUDA's tanh 24, sqrt 8, division 8,
 // reciprocal 5, log 29.75 (inside pow's adjoint) and pow 84.  Each call's device time on the probe agrees with its
 // instruction count within 5 %.  The replay's own sin (or cos) and sincos (fmath.cuh)
-// execute 14 and 17 FP64 instructions (counted in the source; the probe's device time
-// per call, 16.7 and 19.5 DFMA with the chain's add, agrees).  The roofline divides
+// execute 14 and 17 FP64 instructions (counted in the source).  The roofline divides
 // this work by the FP64 pipe's peak issue rate.
 #pragma once
 #include "tape.h"

@@ -1,6 +1,10 @@
 // Tape replay on the GPU (sm_103a): forward sweep, reverse adjoint sweep and
 // per-lane loss for a population of parameter lanes (paper sections 3.4-3.5,
-// Appendix C).
+// Appendix C).  The general kernel: it runs every tape.  Tapes that translate to compact
+// records (compact.h) run on scalar.cu and matrix.cu instead; what stays here is a data axis
+// with matrices in it, loops of more records than shared memory holds, lanes whose slots alone
+// fill a block's shared memory (64-state filters), and the shapes for which capi.cpp finds
+// this kernel faster.
 //
 // Execution model.  Every lane runs the same instruction stream (the tape is
 // shared by the population), so instruction fetch and dispatch are uniform across

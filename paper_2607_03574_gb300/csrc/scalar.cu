@@ -19,9 +19,11 @@
 // record; one warp per scheduler, so the rest is each record's own latency); an exponential
 // fit, 50,001 lanes x 333 points in binary32, 1.33 -> 0.168 (what binds then is issue and the
 // shared-memory bandwidth of 16-byte slots); 24 random expressions x 4096 lanes x 256 points in
-// binary64 on 8 streams, 2.65 -> 2.30 (the FP64 pipe).  Tried and slower on the logistic tape:
+// binary64 on 8 streams, 2.65 -> 2.14 (the FP64 pipe; fmath.cuh's shorter functions are 0.16 of
+// it).  Tried and slower on the logistic tape:
 // two records per dispatch, independent or with the second reading the first's result from
-// a register (2.23 binary64), and no reading ahead of the next record (2.48).
+// a register (2.23 binary64), no reading ahead of the next record (2.48), and record kinds of
+// their own for gated or saved arithmetic (2.14).
 #include "interp.cuh"
 
 namespace ndvm {
