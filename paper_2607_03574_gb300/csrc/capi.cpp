@@ -610,9 +610,14 @@ struct Member {
 // Launches the members in as few kernels as possible: one per run of members with the
 // same kernel variant, block size and threads per lane.  The launch's shared memory is its largest
 // member's, which may cost the others resident blocks: members of different resident blocks per
-// SM share a launch as long as all of its blocks are on the SMs at once.  (24 programs x 64 lanes:
-// two launches instead of seven, one after the other, of which none filled the chip.)  At most
-// kMultiMax members and 2^31 - 1 blocks per launch.
+// SM share a launch while it has at most kMergeRounds times the blocks that are on the SMs at once.
+// Launches follow each other on the stream, and each ends with its slowest blocks on a nearly idle
+// chip; blocks of one launch follow each other without that, the longest programs' first.
+// Random expressions, us per call with one round, two, four, sixteen: 24 programs x 300 lanes x 256
+// points 298, 274, 261, 263; 8 x 1000 x 256 290, 257, 248, 228; 16 x 2000 x 128 570, 510, 467, 441;
+// 30 x 700 x 200 700, 613, 614, 703; 24 x 4096 x 256 2690, 2537, 2503, 2655.  At most kMultiMax
+// members and 2^31 - 1 blocks per launch.
+constexpr int64_t kMergeRounds = 4;
 ndvm_status launch_members(std::vector<Member>& ms, bool f32, void* stream) {
   std::stable_sort(ms.begin(), ms.end(), [](const Member& x, const Member& y) { return x.key < y.key; });
   // (within a kind, fewest resident blocks -- most shared memory -- first)
@@ -621,10 +626,13 @@ ndvm_status launch_members(std::vector<Member>& ms, bool f32, void* stream) {
     int64_t blocks = 0;
     size_t j = i;
     for (; j < ms.size() && std::equal(k.begin(), k.end() - 1, ms[j].key.begin()); j++) {
-      if (ms[j].key != k && blocks + ms[j].blocks > num_sms() * k.back()) break;
+      if (ms[j].key != k && blocks + ms[j].blocks > kMergeRounds * num_sms() * k.back()) break;
       blocks += ms[j].blocks;
     }
     for (size_t q = i; q < j; q++) ms[q].key = k;
+    // (the longest programs' blocks start first)
+    std::stable_sort(ms.begin() + (int64_t)i, ms.begin() + (int64_t)j,
+                     [](const Member& x, const Member& y) { return x.a.n_code > y.a.n_code; });
     i = j;
   }
   std::unique_ptr<MultiArgs> table(new MultiArgs);  // about 31 KB: on the heap

@@ -93,3 +93,22 @@ def test_compact_programs(ndvm, cuda, monkeypatch, make, dtype):
         rel = np.linalg.norm(fast[1] - general[1]) / max(np.linalg.norm(general[1]), 1e-30)
         ok, rep = rel < 2e-5 and np.allclose(fast[0], general[0], rtol=2e-5), rel
     assert ok, rep
+
+
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+@pytest.mark.parametrize("lanes", [[300] * 14, [2000, 1, 900, 4000, 33] * 2, [20000, 15000, 40]])
+def test_batches_past_the_resident_blocks(ndvm, cuda, lanes, dtype):
+    """Members share a launch of more blocks than the GPU holds at once, ordered by length: the same
+    bits as separate calls."""
+    import torch
+    ws = W.random_exprs(len(lanes), B=2, n_points=70, seed=99)
+    tapes = [ndvm.trace_build(w.program, w.frontend) for w in ws]
+    dt = getattr(torch, dtype)
+    params = [torch.tensor(w.params[:1].repeat(n, 0) + 1e-4 * np.arange(n)[:, None], dtype=dt, device=cuda)
+              for w, n in zip(ws, lanes)]
+    obs = [torch.tensor(w.obs, dtype=dt, device=cuda) for w in ws]
+    loss, grad = ndvm.value_and_grad_multi(tapes, params, obs)
+    for t, p, o, l, g in zip(tapes, params, obs, loss, grad):
+        l1, g1 = ndvm.value_and_grad(t, p, o)
+        np.testing.assert_array_equal(l.cpu().numpy(), l1.cpu().numpy())
+        np.testing.assert_array_equal(g.cpu().numpy(), g1.cpu().numpy())
