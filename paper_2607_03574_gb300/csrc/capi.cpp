@@ -231,10 +231,9 @@ bool compact_shape(const Plan& p, size_t elem, int64_t B, Shape* out) {
   const int64_t sms = num_sms();
   const size_t records = p.compact.size() / kCompactWords;
   const bool axis = p.compact_points > 0;
-  // up to kCResident records are held in shared memory whole; longer streams are read in
-  // chunks, which loops do not allow (the general kernels run those)
+  // up to kCResident records are held in shared memory whole; longer streams, which have no
+  // loops (compact_plan leaves those to the general kernels), are read in chunks
   const bool chunked = records > kCResident;
-  if (chunked && axis) return false;
   s.points = 1;
   if (axis && p.n_save == 0) {
     int g = threads_per_lane_override();

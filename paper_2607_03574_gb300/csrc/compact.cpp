@@ -899,7 +899,10 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
   }
   if (code.empty()) return;
   share_reciprocals(code, &p.compact_slots);
-  if (p.compact_points == 0 && code.size() > kCResident) mark_chunks<CRec, kCChunk>(code);
+  // (a loop is not read in chunks, nor is one of no points, which still has its records)
+  const bool loop = std::any_of(code.begin(), code.end(), [](const CRec& c) { return (c.w[0] & 0xff) == C_LOOP; });
+  if (loop && code.size() > kCResident) return;
+  if (code.size() > kCResident) mark_chunks<CRec, kCChunk>(code);
   for (const CRec& c : code) p.compact.insert(p.compact.end(), c.w, c.w + kCompactWords);
 }
 

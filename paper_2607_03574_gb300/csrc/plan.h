@@ -158,7 +158,8 @@ struct Plan {
   // and element-split kernel variants; the plain variant runs `code`)
   std::vector<DInst> code_paired;
   // the stream's compact records (compact.h), kCompactWords words each, for the scalar
-  // kernels; empty when an instruction has no compact form
+  // kernels; empty when an instruction has no compact form, or a stream with a data-axis loop
+  // (of any number of points, 0 included) has more records than shared memory holds
   std::vector<uint32_t> compact;
   int32_t compact_slots = 0;   // slots of the compact form
   int64_t compact_points = 0;  // points of its largest data-axis region (0: none)

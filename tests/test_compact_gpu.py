@@ -54,6 +54,20 @@ def test_compact_equals_general(ndvm, oracle_mod, cuda, monkeypatch, B, n, dtype
         assert ok, rep
 
 
+@pytest.mark.parametrize("steps", [3, 700])
+def test_no_points_beside_a_long_stream(ndvm, cuda, monkeypatch, steps):
+    """A data sum over no points in a stream of more records than shared memory holds."""
+    import torch
+    rng = np.random.default_rng(steps)
+    text = ("(model (params a b) (+ (data-sum 0 1 (* a (dobs 0)))"
+            f" (let loop ((i 0) (x a)) (if (= i {steps}) x (loop (+ i 1) (+ (* x b) (sin x)))))))")
+    w = W.Workload("no_points", text, 0, rng.uniform(-0.5, 0.5, (70, 2)), np.zeros(1), np.zeros(2))
+    fast, general = _both(ndvm, w, torch.float64, monkeypatch)
+    ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-12)
+    assert ok, rep
+    np.testing.assert_array_equal(fast[0], fast[2])
+
+
 def _special():
     """Lanes of zeros, infinities, NaN, subnormals and the largest values through every scalar rule."""
     s = np.array([0.0, -0.0, 1.0, -1.0, np.inf, -np.inf, np.nan, 5e-324, -1e-310, 1e-8, 1.7e308, -3.0, 709.0, 1e6])
