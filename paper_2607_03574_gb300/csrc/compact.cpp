@@ -63,6 +63,7 @@ struct Matrices {
   std::vector<int32_t> lists;
   std::vector<Stage> stages;
   int rev_begin = -1;  // first record of the reverse sweep
+  int temps = 1;       // slots for parameters that are operands: a record's two have one each
 
   int constants(const std::vector<double>& pool, int32_t idx, int width) {
     auto it = runs_.find({idx, width});
@@ -361,8 +362,10 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
               flags |= const_flag;
               return (uint32_t)mx->constants(pool, ref_index(ref), width);
             case RK_PARAM: {
-              const int32_t tmp = p.n_slots + kCExtraSlots;  // (a scalar: one temporary slot)
               if (width != 1) break;
+              const int second = field & 1;  // (of the fields 2 and 3, or 5 and 6)
+              mx->temps = std::max(mx->temps, 1 + second);
+              const int32_t tmp = p.n_slots + kCExtraSlots + second;
               load(mkref(RK_SLOT, tmp), ref);
               return slot(tmp);
             }
@@ -884,7 +887,7 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
     for (const MRec& c : code)
       if ((c.w[0] & 0xff) >= M_F && (c.w[0] & 0xff) <= M_RSELECT)
         p.matrix_width = std::max(p.matrix_width, (int32_t)((c.w[4] & 0xff) * ((c.w[4] >> 8) & 0xff)));
-    p.matrix_slots = place_stages(code, mx, p.n_slots + kCExtraSlots + 1);
+    p.matrix_slots = place_stages(code, mx, p.n_slots + kCExtraSlots + mx.temps);
     mark_chunks<MRec, kMChunk>(code);
     for (const MRec& c : code) p.matrix.insert(p.matrix.end(), c.w, c.w + kMatrixWords);
     p.matrix_consts = mx.consts;

@@ -26,7 +26,7 @@ def sims(tmp_path_factory):
         pytest.skip("no C++ compiler")
     out = tmp_path_factory.mktemp("recsim")
     for name, srcs in (("plansim", PLANNER), ("recsim", PLANNER + ["compact.cpp"])):
-        subprocess.run([cxx, "-O2", "-std=c++17", "-I", CSRC, os.path.join(ROOT, "tests", name + ".cpp"),
+        subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, os.path.join(ROOT, "tests", name + ".cpp"),
                         *[os.path.join(CSRC, f) for f in srcs], "-o", str(out / name)], check=True)
     return out
 
@@ -101,3 +101,16 @@ def test_a_stream_with_a_loop_is_not_cut_into_chunks(sims, n, steps, kind):
     assert agree(sims, w) == [kind, kind]
     alone = program(f"(model (params a b) {LONG.format(start='a', steps=steps)})", 2)
     assert agree(sims, alone) == ["compact", "compact"]
+
+
+ONE_BY_ONE = {  # scalars are 1 x 1 matrices: a record's two operands may both be parameters
+    "m+": "(m+ a b)", "m-": "(m- a b)", "mscale": "(mscale a b)", "matmul": "(matmul a b)", "one": "(matmul a a)",
+    "fold": "(m+ b (matmul a b))", "const": "(m- (mscale 3.0 b) (m+ a 2.0))", "inv": "(matmul (inv a) b)",
+    "det": "(mscale (det a) (logdet (mscale 2.0 (matmul b b))))",
+}
+
+
+@pytest.mark.parametrize("name", sorted(ONE_BY_ONE))
+def test_parameters_as_matrix_operands(sims, name):
+    w = program(f"(model (params a b) (let* ((Z {ONE_BY_ONE[name]})) (+ (* Z Z) (trace (mscale Z b)))))", 2)
+    assert agree(sims, w) == ["matrix", "matrix"]
