@@ -424,6 +424,12 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
                   }
                   most = std::max(most, m);
                 }
+                // (both operands constant: an infinity or a NaN in the other one is no stored value that
+                // the kernel would have met, and binary32 has more infinities; zeros times them count)
+                if (side ? cx : cy) {
+                  const int32_t oat = ref_index(side ? X : Y);
+                  for (int e = 0; e < (side ? wx : wy); e++) finite = finite && std::isfinite((float)pool_at(oat, e));
+                }
                 if (!finite || most >= best) continue;
                 best = most;
                 const bool select = most == 1 && unit && !(more & kMAcc) && !(side ? cx : cy);

@@ -6,8 +6,8 @@
 //
 // Input on stdin:  frontend B P n_obs stream(0 gradient plan, 1 value plan) K / B*P params /
 //                  n_obs obs / the program text up to end of input.
-// Output: the kind of the stream (compact, matrix or none), then one line per lane: the loss and the
-// P gradient components as C hex floats.  Exit status 5: a record failed a check.
+// Output: the kind of the stream (compact, matrix or none) and the entries of its lists, then one line
+// per lane: the loss and the P gradient components as C hex floats.  Exit status 5: a record failed a check.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -692,7 +692,7 @@ int main() {
     Plan p = make_plan(b.t, stream == 0);
     compact_plan(p, b.t.consts);
     check(p, b.t.consts.size() + p.extra_consts.size());
-    std::printf("%s\n", !p.matrix.empty() ? "matrix" : !p.compact.empty() ? "compact" : "none");
+    std::printf("%s %zu\n", !p.matrix.empty() ? "matrix" : !p.compact.empty() ? "compact" : "none", p.matrix_lists.size());
     if (p.matrix.empty() && p.compact.empty()) return 0;
     if (p.n_save > 0 || !p.matrix.empty() || p.compact_points == 0) K = 1;
     std::vector<double> consts = b.t.consts;

@@ -51,7 +51,8 @@ def agree(sims, w, tol=1e-11, B=4):
     for value_plan in (0, 1):
         want = _rows(_run(sims / "plansim", "2" if value_plan else "0", w, B))
         for K in (1, 2, 4):
-            kind, _, rows = _run(sims / "recsim", f"{value_plan} {K}", w, B).partition("\n")
+            head, _, rows = _run(sims / "recsim", f"{value_plan} {K}", w, B).partition("\n")
+            kind = head.split()[0]
             if K == 1:
                 kinds.append(kind)
             if kind == "none":
@@ -114,3 +115,15 @@ ONE_BY_ONE = {  # scalars are 1 x 1 matrices: a record's two operands may both b
 def test_parameters_as_matrix_operands(sims, name):
     w = program(f"(model (params a b) (let* ((Z {ONE_BY_ONE[name]})) (+ (* Z Z) (trace (mscale Z b)))))", 2)
     assert agree(sims, w) == ["matrix", "matrix"]
+
+
+@pytest.mark.parametrize("big,lists", [("1e999", False), ("-1e999", False), ("1e39", False), ("1e38", True)])
+@pytest.mark.parametrize("order", ["(matmul S D)", "(matmul D S)"])
+def test_zeros_of_a_constant_times_an_infinite_constant(sims, order, big, lists):
+    """0 * inf is NaN: a product of two constants leaves out no term when one holds an infinity.  1e39 is
+    one in binary32, whose records have the same lists of the terms to take."""
+    w = program(f"(define S (matrix 2 2 1.5 0.0 0.0 2.0)) (define D (matrix 2 2 {big} 2.0 3.0 4.0))"
+                f"(model (params a b) (trace (mscale a {order})))", 2)
+    assert agree(sims, w) == ["matrix", "matrix"]
+    head = _run(sims / "recsim", "0 1", w, 1).split("\n")[0]
+    assert (int(head.split()[1]) > 0) == lists
