@@ -577,6 +577,7 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
             c.w[1] = slot(f[0]);
             c.w[2] = x;
             c.w[4] = (uint32_t)n;
+            save(c, f[3]);
             break;
           }
           case B_MADD: case B_MSUB:

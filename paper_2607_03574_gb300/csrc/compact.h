@@ -69,7 +69,7 @@ enum COp : uint32_t {
   M_SCALE,      // w1 = w2 (scalar) * w3, w4 elements
   M_INV,        // w1 = inverse of w2, w3 scratch, w4 n | (2^20 / n rounded up) << 8
   M_DET, M_LOGDET,  // w1 of w2, w3 and w4 as above, w5 inverse to slots, w6 inverse to workspace
-  M_TRACE,      // w1 of w2, w4 n
+  M_TRACE,      // w1 of w2, w4 n, w7 save
   M_GATHER,     // w1 = elements named by args[w2 ...], w3 of them
   M_FETCH,      // asynchronous copies of w3 elements from workspace (kMFromObs: observations) w2 on into w1
   M_RSCALE,     // w2 target scalar, w3 target matrix, w5 scalar, w6 matrix, w4 elements

@@ -491,6 +491,7 @@ __device__ __forceinline__ void matrix_rule(const MThread<T>& t, const uint4& r0
       s.v[0] = A[0];
       for (int i = 1; i < n; i++) s.v[0] = s.v[0] + A[i * n + i];
       t.template st<1>(r0.y, s);
+      t.template keep<1>(f, r1.w, s);
       break;
     }
     case M_GATHER: {

@@ -535,7 +535,7 @@ void Planner::emit_forward(int v) {
       }
       break;
     case OP_TRACE:
-      p.d.op = D_TRACE; p.d.r = T.nodes[n.a].rows; p.d.c = 1; p.f[1] = R(ref(n.a));
+      p.d.op = D_TRACE; p.d.r = T.nodes[n.a].rows; p.d.c = 1; p.f[1] = R(ref(n.a)); p.f[3] = save_of(v);
       break;
     default:
       unsupported(std::string("no forward lowering for ") + op_name(n.op));
@@ -1655,7 +1655,7 @@ bool validate_code(const Plan& p, const std::vector<DInst>& code, size_t n_const
         ok = n <= 8 && ref_ok(f[0], 1, true) && ref_ok(f[1], n * n, false) && save_ok(f[3], 1) &&
              ref_ok(f[4], n * n, true) && save_ok(f[5], n * n) && scratch_ok(d);
         break;
-      case D_TRACE: ok = ref_ok(f[0], 1, true) && ref_ok(f[1], n * n, false); break;
+      case D_TRACE: ok = ref_ok(f[0], 1, true) && ref_ok(f[1], n * n, false) && save_ok(f[3], 1); break;
       case D_ZERO: case D_GREDUCE: ok = f[1] >= 0 && ref_ok(f[0], f[1], true); break;
       case D_LOOP:
         ok = open_loop < 0 && f[3] > (int)pc && f[3] < (int)code.size() && code[f[3]].op == D_ENDLOOP &&

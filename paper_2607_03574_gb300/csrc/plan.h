@@ -41,7 +41,7 @@ enum DOp : uint8_t {
   D_MATMUL,         // f0 out, f1 A, f2 B, f3 save; r x c, inner k
   D_INV,            // f0 out, f1 A, f2 scratch (n >= 4), f3 save; n = r
   D_DET, D_LOGDET,  // f0 out, f1 A, f2 scratch (n >= 4), f3 save, f4 aux slot (inverse), f5 aux save; n = r
-  D_TRACE,          // f0 out, f1 A; n = r
+  D_TRACE,          // f0 out, f1 A, f3 save; n = r
   // ---- data-axis regions ----
   D_ZERO,           // f0 slot, f1 count
   D_LOOP,           // f0 N, f1 stride, f2 base, f3 pc of the matching D_ENDLOOP

@@ -609,6 +609,7 @@ __device__ __forceinline__ void replay_body(const ReplayArgs& a, const int block
         T s = A[0];
         for (int i = 1; i < n; i++) s = s + A[i * n + i];
         L.st(f[0], 0, s);
+        L.save_out(f[3], 0, s);
         break;
       }
       // ------------------------------------------------------------ data axis

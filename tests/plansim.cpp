@@ -343,6 +343,7 @@ struct Run {
           double t = el(f[1], 0);
           for (int i = 1; i < n; i++) t = t + el(f[1], i * n + i);
           slot(f[0]) = t;
+          save_out(f[3], t);
           break;
         }
         case B_GATHER: {

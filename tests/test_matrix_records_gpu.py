@@ -106,3 +106,16 @@ def test_banded_constants_sum_as_dense(ndvm, cuda, monkeypatch, n, band, dtype):
     fast, general = _both(ndvm, w, getattr(torch, dtype), monkeypatch)
     for x, y in zip(fast, general):
         np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("steps", [3, 200])
+def test_a_saved_trace(ndvm, oracle_mod, cuda, monkeypatch, steps):
+    """The reverse sweep of a long tape reads a trace from the workspace, on both kernels."""
+    import torch
+    text = ("(model (params a b) (let loop ((i 0) (x a)) (if (= i %d) x (let* ((M (matrix 2 2 x b b a)) (t (trace M)))"
+            " (loop (+ i 1) (sin (* t (* 0.5 x))))))))" % steps)
+    w = W.Workload("trace", text, 0, np.random.default_rng(steps).normal(0.3, 0.7, (70, 2)), np.zeros(1), np.zeros(2))
+    for loss, grad, _ in _both(ndvm, w, torch.float64, monkeypatch):
+        ol, og, sp = oracle_ref(oracle_mod, w.program, w.params, w.obs)
+        ok, rep = rel_check(loss, grad, ol, og, 1e-12, sp)
+        assert ok, rep

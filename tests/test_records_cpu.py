@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import workloads as W
-from conftest import hazard_workloads, matrix_program
+from conftest import hazard_workloads, matrix_program, oracle_ref, rel_check
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2607_03574_gb300", "csrc")
@@ -127,3 +127,18 @@ def test_zeros_of_a_constant_times_an_infinite_constant(sims, order, big, lists)
     assert agree(sims, w) == ["matrix", "matrix"]
     head = _run(sims / "recsim", "0 1", w, 1).split("\n")[0]
     assert (int(head.split()[1]) > 0) == lists
+
+
+TRACES = ("(model (params a b) (let loop ((i 0) (x a)) (if (= i {steps}) x "
+          "(let* ((M (matrix 2 2 x b b a)) (t (trace M))) (loop (+ i 1) (sin (* t (* 0.5 x))))))))")
+
+
+@pytest.mark.parametrize("steps", [3, 200])
+def test_a_trace_that_the_reverse_sweep_reads_is_saved(sims, oracle_mod, steps):
+    """A long tape's forward values reach the reverse sweep through the workspace, a trace's too."""
+    w = program(TRACES.format(steps=steps), 2)
+    assert agree(sims, w) == ["matrix", "matrix"]
+    got = _rows(_run(sims / "plansim", "0", w, w.B))
+    loss, grad, spread = oracle_ref(oracle_mod, w.program, w.params, w.obs)
+    ok, rep = rel_check(got[:, 0], got[:, 1:], loss, grad, 1e-12, spread)
+    assert ok, rep
