@@ -932,6 +932,14 @@ ndvm_status ndvm_value_and_grad_multi(const ndvm_tape* const* tapes, int32_t n_t
 namespace {
 
 // host-buffer replay: copies in, replay, copies out, on one stream; `sync` waits for them
+// Host memory that CUDA does not know.
+bool is_pageable(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeUnregistered;
+  cudaGetLastError();
+  return false;
+}
+
 ndvm_status host_replay(const ndvm_tape* tape, ndvm_dtype dtype, int64_t B, const void* params, const void* obs,
                         int64_t n_obs, void* loss, void* grad, void* stream, bool sync) {
   ndvm_tape* t = const_cast<ndvm_tape*>(tape);
@@ -959,10 +967,12 @@ ndvm_status host_replay(const ndvm_tape* tape, ndvm_dtype dtype, int64_t B, cons
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
   // A synchronous call's small inputs and outputs travel as one copy each way, through a buffer of
-  // this call: a transfer's fixed cost (about 8 us) is more than copying 64 KB on the host
+  // this call: a transfer's fixed cost (about 8 us) is more than copying 64 KB on the host.  Not so
+  // inputs in page-locked or managed memory: earlier work on the stream may still write them, and
+  // copies on the stream come after it.
   constexpr size_t kOneCopy = 64 * 1024;
   std::vector<char> host;
-  if (sync && pb && ob && in <= kOneCopy) {
+  if (sync && pb && ob && in <= kOneCopy && is_pageable(params) && is_pageable(obs)) {
     host.resize(in);
     std::memcpy(host.data(), params, pb);
     std::memcpy(host.data() + pad(pb), obs, ob);

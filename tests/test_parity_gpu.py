@@ -212,6 +212,28 @@ def test_host_entry_point_matches_device(ndvm, cuda):
     np.testing.assert_array_equal(hg, gg)
 
 
+def test_host_inputs_written_by_earlier_work_on_the_stream(ndvm, cuda):
+    """Page-locked inputs are read after the work that is queued on the call's stream before it."""
+    import torch
+    w = W.config(1, B=64)
+    tape = ndvm.trace_build(w.program, w.frontend)
+    want = ndvm.value_and_grad_host(tape, w.params, w.obs)
+    params = torch.zeros(w.params.shape, dtype=torch.float64).pin_memory()
+    obs = torch.zeros(w.obs.size, dtype=torch.float64).pin_memory()
+    dp, do = torch.tensor(w.params, device=cuda), torch.tensor(w.obs, device=cuda)
+    big = torch.ones(4096, 4096, device=cuda)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        for _ in range(20):  # some milliseconds
+            big = big @ big * 1e-4
+        params.copy_(dp, non_blocking=True)
+        obs.copy_(do, non_blocking=True)
+    got = ndvm.value_and_grad_host(tape, params.numpy(), obs.numpy(), stream=s)
+    for a, b in zip(got, want):
+        np.testing.assert_array_equal(a, b)
+
+
 def test_logistic_fp32_variant(ndvm, oracle_mod, cuda):
     """fp32 replay against the oracle in binary32 arithmetic, 1e-5 relative."""
     w = W.logistic(B=300)
