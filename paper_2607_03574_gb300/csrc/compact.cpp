@@ -168,6 +168,7 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
   int loop_pc = -1;           // the open C_LOOP record
   int32_t seed = -1;          // slot of a seed set before the loop being translated
   int32_t pending_seed = -1;  // slot of a seed set just before a loop
+  std::vector<int32_t> seeds;  // slots of the seeds set since the last loop
   struct Known { uint32_t op; int nz, list; uint32_t flags; };
   std::map<std::vector<int32_t>, Known> products;  // by a product's operands and shape
   int32_t last_product = -1;  // slot of the product that the last record computes
@@ -251,6 +252,10 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
       case D_LOOP: {
         if (loop_pc >= 0 || mx) return none;
         seed = pending_seed;
+        // (a seed that the loop's body may read and that is not the points' validity there would
+        // count the points past the last one)
+        for (int32_t s : seeds)
+          if (s != seed) return none;
         MRec& c = rec(C_LOOP, (uint32_t)f[0], (uint32_t)f[1]);
         c.w[3] = (uint32_t)f[2];
         for (const DeriveInfo& di : p.derive_info)
@@ -285,6 +290,7 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
           }
         loop_pc = -1;
         seed = -1;
+        seeds.clear();
         break;
       case D_SEED:
         if (mx && mx->rev_begin < 0) mx->rev_begin = (int)code.size();
@@ -292,6 +298,7 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
           arith(f[0], mkref(RK_SLOT, valid_slot), false, -1, -1, -1, 0);
         } else {
           rec(C_SEED, slot(f[0]));
+          seeds.push_back(f[0]);
           bool before_loop = false;  // only loads and other seeds between it and a loop
           for (size_t q = pc + 1; q < p.code.size(); q++) {
             if (p.code[q].op == D_LOOP) before_loop = true;

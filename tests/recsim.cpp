@@ -6,6 +6,7 @@
 //
 // Input on stdin:  frontend B P n_obs stream(0 gradient plan, 1 value plan) K / B*P params /
 //                  n_obs obs / the program text up to end of input.
+// With the argument "apart", a record that does nothing stands between each seed and its loop.
 // Output: the kind of the stream (compact, matrix or none) and the entries of its lists, then one line
 // per lane: the loss and the P gradient components as C hex floats.  Exit status 5: a record failed a check.
 #include <cmath>
@@ -670,9 +671,31 @@ void check(const Plan& p, size_t n_consts) {
   need(n == 0 || (code[(n - 1) * words] & 0xff) == C_END, "no end record", n);
 }
 
+// an instruction that zeroes no slots ahead of every loop
+void part_seeds(Plan& p) {
+  std::vector<DInst> out;
+  std::vector<int32_t> at;
+  for (const DInst& d : p.code) {
+    if (d.op == D_LOOP) {
+      DInst z;
+      z.op = D_ZERO;
+      z.f[0] = mkref(RK_SLOT, 0);
+      z.f[1] = 0;
+      out.push_back(z);
+    }
+    at.push_back((int32_t)out.size());
+    out.push_back(d);
+  }
+  for (DInst& d : out) {
+    if (d.op == D_LOOP) d.f[3] = at[(size_t)d.f[3]];
+    if (d.op == D_ENDLOOP) d.f[0] = at[(size_t)d.f[0]];
+  }
+  p.code.swap(out);
+}
+
 }  // namespace
 
-int main() {
+int main(int argc, char** argv) {
   int fe = 0, stream = 0, K = 1;
   int64_t B = 0, P = 0, n_obs = 0;
   std::cin >> fe >> B >> P >> n_obs >> stream >> K;
@@ -690,6 +713,7 @@ int main() {
     else trace_bytecode(text.data(), text.size(), b, err);
     if (b.t.loss < 0) { std::fprintf(stderr, "no result: %s\n", err.c_str()); return 2; }
     Plan p = make_plan(b.t, stream == 0);
+    if (argc > 1 && std::string(argv[1]) == "apart") part_seeds(p);
     compact_plan(p, b.t.consts);
     check(p, b.t.consts.size() + p.extra_consts.size());
     std::printf("%s %zu\n", !p.matrix.empty() ? "matrix" : !p.compact.empty() ? "compact" : "none", p.matrix_lists.size());

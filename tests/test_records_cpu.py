@@ -31,10 +31,10 @@ def sims(tmp_path_factory):
     return out
 
 
-def _run(exe, head, w, B):
+def _run(exe, head, w, B, *args):
     env = {k: v for k, v in os.environ.items() if not k.startswith("NDVM_")}
     body = " ".join(repr(float(x)) for x in w.params[:B].ravel()) + "\n" + " ".join(repr(float(x)) for x in w.obs) + "\n"
-    r = subprocess.run([str(exe)], input=f"{w.frontend} {B} {w.P} {w.obs.size} {head}\n{body}{w.program}",
+    r = subprocess.run([str(exe), *args], input=f"{w.frontend} {B} {w.P} {w.obs.size} {head}\n{body}{w.program}",
                        capture_output=True, text=True, env=env, timeout=300)
     assert r.returncode == 0, (w.name, r.stderr)
     return r.stdout
@@ -142,3 +142,12 @@ def test_a_trace_that_the_reverse_sweep_reads_is_saved(sims, oracle_mod, steps):
     loss, grad, spread = oracle_ref(oracle_mod, w.program, w.params, w.obs)
     ok, rep = rel_check(got[:, 0], got[:, 1:], loss, grad, 1e-12, spread)
     assert ok, rep
+
+
+def test_a_seed_apart_from_its_loop_is_refused(sims):
+    """Points past the last one are told by the body's seed, set just ahead of the loop: a stream in which
+    it is not recognised as the loop's has no compact form."""
+    w = program("(model (params a b) (data-sum 3 2 (let ((r (- (* a (exp (* b (dobs 0)))) (dobs 1)))) (* r r))))", 2, 6)
+    assert agree(sims, w) == ["compact", "compact"]
+    kinds = [_run(sims / "recsim", f"{stream} 1", w, 1, "apart").split()[0] for stream in (0, 1)]
+    assert kinds == ["none", "compact"]  # (the value plan's loop has no seed)
