@@ -714,8 +714,8 @@ std::vector<MRec> translate(const Plan& p, const std::vector<double>& consts, in
   return kept;
 }
 
-// The slot that a record writes, when it writes one value (kCNone otherwise); all = false when it
-// may write others too.
+// The slot that a record writes, when it writes one value or none (kCNone); all = false when it may
+// write others.
 uint32_t writes(const CRec& c, bool* all) {
   const uint32_t op = c.w[0] & 0xff;
   *all = true;
@@ -745,10 +745,10 @@ void share_reciprocals(std::vector<CRec>& code, int32_t* n_slots) {
     const uint32_t op = c.w[0] & 0xff;
     if (op == C_LOOP) { loop = true; write(c.w[5], pc); }
     if (op == C_ENDLOOP) loop = false;
-    bool one;
-    const uint32_t s = writes(c, &one);
+    bool all;
+    const uint32_t s = writes(c, &all);
     if (s != kCNone) write(s, pc);
-    if (one || op == C_LOOP || op == C_ENDLOOP) continue;
+    if (all || op == C_LOOP || op == C_ENDLOOP) continue;
     if (op == C_ZERO || op == C_GREDUCE) {
       for (uint32_t e = 0; e < c.w[2]; e++) write(c.w[1] + e * kCSlotUnit, pc);
     } else if (op == C_FETCH || op == C_OBS) {
@@ -777,12 +777,12 @@ void share_reciprocals(std::vector<CRec>& code, int32_t* n_slots) {
     if (op != C_DIV) continue;
     const Use& u = use[c.w[3]];
     if (u.writers != 1 || u.in_loop || u.writer >= pc || (u.divisions < 2 && !loop) || rcp.count(c.w[3])) continue;
+    if ((code[(size_t)u.writer].w[0] & 0xff) == C_FETCH) continue;  // its copy lands later
     if ((int)rcp.size() >= kCMaxReciprocals) break;
     make[u.writer] = c.w[3];
     rcp[c.w[3]] = (uint32_t)(*n_slots)++ * kCSlotUnit;
   }
   if (rcp.empty()) return;
-  std::map<uint32_t, uint32_t> aux;  // a division's own reciprocal slot -> the shared one
   std::vector<CRec> out;
   std::vector<uint32_t> newpc(code.size());
   for (int pc = 0; pc < (int)code.size(); pc++) {
