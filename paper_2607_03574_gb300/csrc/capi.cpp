@@ -817,13 +817,14 @@ ndvm_status ndvm_trace_build(const char* program, size_t len, ndvm_frontend fe, 
     t->tape = std::move(b.t);
     t->grad_plan = make_plan(t->tape, true);
     t->value_plan = make_plan(t->tape, false);
-    compact_plan(t->grad_plan, t->tape.consts);
-    compact_plan(t->value_plan, t->tape.consts);
     std::string why;
     if (!validate_plan(t->grad_plan, t->tape.consts.size(), why) || !validate_plan(t->value_plan, t->tape.consts.size(), why)) {
       delete t;
       return fail(NDVM_E_UNSUPPORTED, "internal plan check failed: " + why);
     }
+    // (of checked plans: the translation indexes their lists and constants)
+    compact_plan(t->grad_plan, t->tape.consts);
+    compact_plan(t->value_plan, t->tape.consts);
     *out = t;
     return NDVM_OK;
   } catch (const BuildError& e) {
