@@ -222,9 +222,10 @@ int ilog2(int g) {
   return l;
 }
 
-// The launch shape of a compact stream; false when it does not fit.  Threads per lane and
-// points per thread depend on the lanes and the points alone, so that a tape's value and
-// gradient plans sum in the same order.
+// The launch shape of a compact stream; false when it does not fit.  Without a workspace, threads per
+// lane and points per thread depend on the lanes and the points alone, so that a tape's value and
+// gradient plans sum in the same order (tape_shape).  A gradient plan with a workspace takes the
+// points one by one; its value plan, which has none, splits them, and sums in another order.
 bool compact_shape(const Plan& p, size_t elem, int64_t B, Shape* out) {
   if (p.compact.empty()) return false;
   Shape s;
@@ -466,6 +467,20 @@ Shape launch_shape(const Plan& p, size_t elem, int64_t B) {
   return s;
 }
 
+// The same of a tape's gradient or value plan.  A data sum's points are added in the order of the
+// kernel that runs them, so the value plan runs on the general one where the gradient plan's slots do
+// not fit the other.
+Shape tape_shape(const ndvm_tape* t, bool grad, size_t elem, int64_t B) {
+  const Plan &g = t->grad_plan, &v = t->value_plan;
+  Shape s = launch_shape(grad ? g : v, elem, B);
+  if (!grad && s.points && v.compact_points > 0 && g.n_save == 0 && !launch_shape(g, elem, B).points) {
+    const int chunk_lanes = s.chunk_lanes;
+    s = general_shape(v, elem, B);
+    s.chunk_lanes = chunk_lanes;
+  }
+  return s;
+}
+
 // bytes of the extended observations (a copy of the observations the program reads,
 // then the regions' blocks of shared per-point values), rounded up to 256; 0 without
 size_t derived_bytes(const Plan& p, size_t elem) {
@@ -534,7 +549,7 @@ ndvm_status run(ndvm_tape* t, bool grad, ndvm_dtype dtype, int64_t B, const void
   if (n_obs < p.n_obs_min) return fail(NDVM_E_INVALID_ARG, "obs holds " + std::to_string(n_obs) + " values but the program reads " + std::to_string(p.n_obs_min));
   if (p.n_obs_min > 0 && !obs) return fail(NDVM_E_INVALID_ARG, "null obs");
   const size_t elem = dtype == NDVM_F32 ? sizeof(float) : sizeof(double);
-  const Shape sh = launch_shape(p, elem, B);
+  const Shape sh = tape_shape(t, grad, elem, B);
   const int tpb = sh.tpb, log2g = sh.log2g;
   const size_t smem = sh.smem;
   if (smem > kSmemLimit) return fail(NDVM_E_UNSUPPORTED, "tape needs " + std::to_string(p.n_slots) + " slots per lane, more than shared memory holds");
@@ -825,6 +840,12 @@ ndvm_status ndvm_trace_build(const char* program, size_t len, ndvm_frontend fe, 
     // (of checked plans: the translation indexes their lists and constants)
     compact_plan(t->grad_plan, t->tape.consts);
     compact_plan(t->value_plan, t->tape.consts);
+    // (both or neither, where both split a data sum's points: its order of addition is the kernel's)
+    Plan &g = t->grad_plan, &v = t->value_plan;
+    if (g.has_regions && g.n_save == 0 && g.compact.empty() != v.compact.empty()) {
+      g.compact.clear();
+      v.compact.clear();
+    }
     *out = t;
     return NDVM_OK;
   } catch (const BuildError& e) {

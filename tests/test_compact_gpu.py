@@ -68,6 +68,23 @@ def test_no_points_beside_a_long_stream(ndvm, cuda, monkeypatch, steps):
     np.testing.assert_array_equal(fast[0], fast[2])
 
 
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+@pytest.mark.parametrize("terms,values", [(20, 1), (165, 1), (20, 70), (20, 75)])
+def test_value_and_gradient_plans_add_in_the_same_order(ndvm, cuda, terms, values, dtype):
+    """The second and the last body's gradient stream alone is too long for the compact form: the value
+    plan then runs on the general kernel as well, and the loss keeps its bits."""
+    import torch
+    rng = np.random.default_rng(terms)
+    u = " ".join(f"(v{i} (sin (* {0.1 + 0.01 * i} (* b x))))" for i in range(values))
+    t = " ".join(f"(* v{i % values} (+ a (* {0.5 + i} x)))" for i in range(max(terms, values)))
+    text = (f"(model (params a b) (data-sum 301 2 (let* ((x (dobs 0)) {u} (r (- (+ {t}) (dobs 1)))) (* r r))))")
+    tape = ndvm.trace_build(text)
+    p = torch.tensor(rng.normal(size=(300, 2)), dtype=getattr(torch, dtype), device=cuda)
+    o = torch.tensor(rng.normal(size=602), dtype=getattr(torch, dtype), device=cuda)
+    loss, _ = ndvm.value_and_grad(tape, p, o)
+    np.testing.assert_array_equal(ndvm.forward(tape, p, o).cpu().numpy(), loss.cpu().numpy())
+
+
 def _special():
     """Lanes of zeros, infinities, NaN, subnormals and the largest values through every scalar rule."""
     s = np.array([0.0, -0.0, 1.0, -1.0, np.inf, -np.inf, np.nan, 5e-324, -1e-310, 1e-8, 1.7e308, -3.0, 709.0, 1e6])
