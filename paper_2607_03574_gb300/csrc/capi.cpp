@@ -772,21 +772,25 @@ ndvm_status run_multi(ndvm_tape* const* tapes, int32_t n, ndvm_dtype dtype, cons
         der.push_back(m);
       }
     }
-    Member m(shapes[(size_t)k]);
-    ReplayArgs& a = m.a;
-    plan_args(a, p, dp, m.sh, dtype, dc->err);
-    set_obs(a, m.sh, obs[k], der_bytes > 0 ? base : nullptr);
-    a.params = params[k];
-    a.loss = loss[k];
-    a.grad = grad[k];
-    a.save = base + der_bytes;
-    a.save_ld = B[k];
-    a.lane0 = 0;
-    a.lane_end = B[k];
-    const int64_t lpb = m.sh.tpb >> m.sh.log2g;
-    m.blocks = (B[k] + lpb - 1) / lpb;
-    if (m.blocks > 0x7fffffff) return fail(NDVM_E_INVALID_ARG, "too many lanes for one launch");
-    main.push_back(m);
+    // (members of at most kMaxChunk lanes where they use the workspace, each a part of its own)
+    const int64_t chunk = p.n_save > 0 ? std::min(B[k], kMaxChunk) : B[k];
+    for (int64_t l0 = 0; l0 < B[k]; l0 += chunk) {
+      Member m(shapes[(size_t)k]);
+      ReplayArgs& a = m.a;
+      plan_args(a, p, dp, m.sh, dtype, dc->err);
+      set_obs(a, m.sh, obs[k], der_bytes > 0 ? base : nullptr);
+      a.params = params[k];
+      a.loss = loss[k];
+      a.grad = grad[k];
+      a.lane0 = l0;
+      a.lane_end = std::min(l0 + chunk, B[k]);
+      const int64_t lanes = a.lane_end - l0, lpb = m.sh.tpb >> m.sh.log2g;
+      a.save = base + der_bytes + (size_t)l0 * (size_t)p.n_save * elem;
+      a.save_ld = lanes;
+      m.blocks = (lanes + lpb - 1) / lpb;
+      if (m.blocks > 0x7fffffff) return fail(NDVM_E_INVALID_ARG, "too many lanes for one launch");
+      main.push_back(m);
+    }
   }
   if (runs->n > 0) run_batches.push_back(*runs);
   for (const CopyRuns& c : run_batches) {

@@ -110,3 +110,19 @@ def test_batched_argument_errors(ndvm, cuda):
     with pytest.raises(ndvm.NdvmError, match="tape 1"):
         ndvm.value_and_grad_multi(tapes, params, [obs[0], obs[1][:3]])
     assert ndvm.launch_count() == before
+
+
+@pytest.mark.parametrize("extra", [1, 77])
+def test_more_lanes_than_a_part_of_the_workspace_holds(ndvm, cuda, extra):
+    """Lanes that use the workspace run in parts of 2^22, each with a part of the workspace."""
+    import torch
+    text = "(model (params a b) (let loop ((i 0) (x a)) (if (= i 150) x (loop (+ i 1) (+ (* x b) (sin x))))))"
+    tape = ndvm.trace_build(text)
+    B = (1 << 22) + extra
+    assert tape.workspace_bytes(B) > 0
+    p = torch.linspace(-0.5, 0.5, 2 * B, dtype=torch.float32, device=cuda).reshape(B, 2)
+    o = torch.zeros(1, dtype=torch.float32, device=cuda)
+    loss, grad = ndvm.value_and_grad_multi([tape], [p], [o])
+    for rows in (slice(0, 300), slice(B // 2, B // 2 + 300), slice((1 << 22) - 150, B)):
+        l1, g1 = ndvm.value_and_grad(tape, p[rows].contiguous(), o)
+        assert torch.equal(loss[0][rows], l1) and torch.equal(grad[0][rows], g1)
