@@ -876,8 +876,9 @@ ndvm_status ndvm_tape_cost(const ndvm_tape* t, double* work_fwd, double* work_re
                            int32_t* flags) {
   if (!t) return fail(NDVM_E_INVALID_ARG, "null tape");
   const Plan& p = t->grad_plan;
-  if (work_fwd) *work_fwd = p.work_fwd;
-  if (work_rev) *work_rev = p.work_rev;
+  const bool records = !p.compact.empty() || !p.matrix.empty();
+  if (work_fwd) *work_fwd = p.work_fwd + (records ? p.records_fwd : 0);
+  if (work_rev) *work_rev = p.work_rev + (records ? p.records_rev : 0);
   if (save_elems) *save_elems = p.n_save;
   if (flags) *flags = (p.has_regions ? 1 : 0) | (p.spill ? 2 : 0);
   return NDVM_OK;

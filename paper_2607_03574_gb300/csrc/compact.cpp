@@ -7,6 +7,8 @@
 #include <cstring>
 #include <map>
 
+#include "cost.h"
+
 namespace ndvm {
 namespace {
 
@@ -808,6 +810,25 @@ void share_reciprocals(std::vector<CRec>& code, int32_t* n_slots) {
   code.swap(out);
 }
 
+// What the divisions that the records run add to the plan's work (less than 0): the planner counts a lane-level one as
+// the IEEE division and a body's with a reciprocal of its own, kept for the reverse rule; here
+// every division is by a reciprocal, shared or its own.
+template <typename R>
+void recount_divisions(Plan& p, const std::vector<R>& code) {
+  const double whole = cost::kRcpNewton + cost::kDivStep;
+  double points = 1;
+  bool loop = false;
+  p.records_fwd = p.records_rev = 0;
+  for (const R& c : code) {
+    const uint32_t op = c.w[0] & 0xff;
+    if (op == C_LOOP) { loop = true; points = (double)c.w[1]; }
+    if (op == C_ENDLOOP) { loop = false; points = 1; }
+    if (op == C_RCP) p.records_fwd += points * cost::kRcpNewton;
+    if (op == C_DIV) p.records_fwd += points * ((c.w[4] != kCNone ? cost::kDivStep : whole) - (loop ? whole : cost::kDiv));
+    if (op == R_DIV) p.records_rev += points * ((c.w[7] != kCNone ? cost::kDivStep : whole) - (loop ? cost::kDivStep : cost::kDiv));
+  }
+}
+
 // Inserts the staged operands' copies and waits, and gives them slots from `slots` on; returns
 // the slots in use.
 int place_stages(std::vector<MRec>& code, Matrices& mx, int slots) {
@@ -901,6 +922,7 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
     for (const MRec& c : code)
       if ((c.w[0] & 0xff) >= M_F && (c.w[0] & 0xff) <= M_RSELECT)
         p.matrix_width = std::max(p.matrix_width, (int32_t)((c.w[4] & 0xff) * ((c.w[4] >> 8) & 0xff)));
+    recount_divisions(p, code);
     p.matrix_slots = place_stages(code, mx, p.n_slots + kCExtraSlots + mx.temps);
     mark_chunks<MRec, kMChunk>(code);
     for (const MRec& c : code) p.matrix.insert(p.matrix.end(), c.w, c.w + kMatrixWords);
@@ -919,6 +941,7 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
   // (a loop is not read in chunks, nor is one of no points, which still has its records)
   const bool loop = std::any_of(code.begin(), code.end(), [](const CRec& c) { return (c.w[0] & 0xff) == C_LOOP; });
   if (loop && code.size() > kCResident) return;
+  recount_divisions(p, code);
   if (code.size() > kCResident) mark_chunks<CRec, kCChunk>(code);
   for (const CRec& c : code) p.compact.insert(p.compact.end(), c.w, c.w + kCompactWords);
 }

@@ -115,7 +115,7 @@ constexpr int kCSlotValid = 0, kCSlotOne = 1, kCSlotMinusZero = 2, kCExtraSlots 
 
 // Sets p.compact, p.compact_slots and p.compact_points (and its derive plans') from p.code and
 // the constant pool (the tape's `consts`, then p.extra_consts); p.compact stays empty when the
-// stream has an instruction without a compact form.
+// stream has an instruction without a compact form.  Sets the records' work.
 // For a tape with matrices and no data axis, the same for p.matrix*.
 void compact_plan(Plan& p, const std::vector<double>& consts);
 

@@ -152,6 +152,12 @@ def test_cost_model_counts(ndvm):
     c = ndvm.trace_build("(model (params a b) (+ (* a b) a))").cost()
     # forward mul + add; reverse: add copies into its first targets, mul contributes two products
     assert c["work_fwd"] == 2 and c["work_rev"] == 2
+    # divisions by one value, and their adjoints, share its reciprocal (3); each is then 3
+    c = ndvm.trace_build("(model (params a b c) (+ (/ a c) (/ b c)))").cost()
+    # reverse: a's and b's quotients, and -q z into c's adjoint twice
+    assert c["work_fwd"] == 3 + 2 * 3 + 1 and c["work_rev"] == 2 * 3 + 2
+    c = ndvm.trace_build("(model (params a b) (/ a b))").cost()
+    assert c["work_fwd"] == 3 + 3 and c["work_rev"] == 3 + 1
     lg = ndvm.trace_build(W.logistic(B=1).program, ndvm.FE_BYTECODE)
     assert lg.cost()["spill"] and lg.workspace_bytes(10) == lg.cost()["save_elems"] * 8 * 10
     assert lg.workspace_bytes(10, ndvm.F32) == lg.cost()["save_elems"] * 4 * 10
