@@ -810,22 +810,35 @@ void share_reciprocals(std::vector<CRec>& code, int32_t* n_slots) {
   code.swap(out);
 }
 
-// What the divisions that the records run add to the plan's work (less than 0): the planner counts a lane-level one as
-// the IEEE division and a body's with a reciprocal of its own, kept for the reverse rule; here
-// every division is by a reciprocal, shared or its own.
+// What the records add to the plan's work (less than 0).  The planner counts a lane-level division as
+// the IEEE division and a body's with a reciprocal of its own, kept for the reverse rule; here every
+// division is by a reciprocal, shared or its own.  And it counts every term of a product or of a
+// scaling's adjoint; here the terms of a constant's zeros are left out, and a selection has none.
 template <typename R>
-void recount_divisions(Plan& p, const std::vector<R>& code) {
+void recount(Plan& p, const std::vector<R>& code, const Matrices* mx) {
   const double whole = cost::kRcpNewton + cost::kDivStep;
   double points = 1;
   bool loop = false;
   p.records_fwd = p.records_rev = 0;
   for (const R& c : code) {
-    const uint32_t op = c.w[0] & 0xff;
-    if (op == C_LOOP) { loop = true; points = (double)c.w[1]; }
+    const uint32_t* w = c.w;
+    const uint32_t op = w[0] & 0xff;
+    if (op == C_LOOP) { loop = true; points = (double)w[1]; }
     if (op == C_ENDLOOP) { loop = false; points = 1; }
     if (op == C_RCP) p.records_fwd += points * cost::kRcpNewton;
-    if (op == C_DIV) p.records_fwd += points * ((c.w[4] != kCNone ? cost::kDivStep : whole) - (loop ? whole : cost::kDiv));
-    if (op == R_DIV) p.records_rev += points * ((c.w[7] != kCNone ? cost::kDivStep : whole) - (loop ? cost::kDivStep : cost::kDiv));
+    if (op == C_DIV) p.records_fwd += points * ((w[4] != kCNone ? cost::kDivStep : whole) - (loop ? whole : cost::kDiv));
+    if (op == R_DIV) p.records_rev += points * ((w[7] != kCNone ? cost::kDivStep : whole) - (loop ? cost::kDivStep : cost::kDiv));
+    if (op >= M_FSPARSE && op <= M_RSELECT && (w[0] & (kMConstX | kMConstY))) {
+      const uint32_t e = (w[4] & 0xff) * ((w[4] >> 8) & 0xff), K = (w[4] >> 16) & 0xff;
+      double terms = 0;
+      for (uint32_t q = 0; op <= M_RSPARSE && q < e * (w[4] >> 24); q++) {
+        const uint32_t x = (uint32_t)mx->lists[w[8] + q];
+        terms += x != kCNone && x != kMSplit;
+      }
+      (op == M_FSPARSE || op == M_SELECT ? p.records_fwd : p.records_rev) += terms - (double)e * K;
+    }
+    if (op == M_RSCALE && w[2] != kCNone && (w[0] & kMConstY))
+      for (uint32_t q = 0; q < w[4]; q++) p.records_rev -= mx->consts[w[6] + q] == 0;
   }
 }
 
@@ -922,7 +935,7 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
     for (const MRec& c : code)
       if ((c.w[0] & 0xff) >= M_F && (c.w[0] & 0xff) <= M_RSELECT)
         p.matrix_width = std::max(p.matrix_width, (int32_t)((c.w[4] & 0xff) * ((c.w[4] >> 8) & 0xff)));
-    recount_divisions(p, code);
+    recount(p, code, &mx);
     p.matrix_slots = place_stages(code, mx, p.n_slots + kCExtraSlots + mx.temps);
     mark_chunks<MRec, kMChunk>(code);
     for (const MRec& c : code) p.matrix.insert(p.matrix.end(), c.w, c.w + kMatrixWords);
@@ -941,7 +954,7 @@ void compact_plan(Plan& p, const std::vector<double>& consts) {
   // (a loop is not read in chunks, nor is one of no points, which still has its records)
   const bool loop = std::any_of(code.begin(), code.end(), [](const CRec& c) { return (c.w[0] & 0xff) == C_LOOP; });
   if (loop && code.size() > kCResident) return;
-  recount_divisions(p, code);
+  recount(p, code, nullptr);
   if (code.size() > kCResident) mark_chunks<CRec, kCChunk>(code);
   for (const CRec& c : code) p.compact.insert(p.compact.end(), c.w, c.w + kCompactWords);
 }

@@ -24,8 +24,9 @@ constexpr double kExp = 7, kLog = 11, kSin = 14, kSinCos = 17, kTanh = 24, kSqrt
 // two fused multiply-adds, kDivStep); its reverse rule divides the adjoint by b with the
 // forward sweep's reciprocal (kDivStep).  A lane-level division is the IEEE division
 // (kDiv) in both sweeps on the general kernel; on the others it is counted as their records
-// run it, by a reciprocal that divisions by the same value share (recount_divisions in
-// compact.cpp).  The log's adjoint divides the same way as a body division.
+// run it, by a reciprocal that divisions by the same value share (recount in compact.cpp,
+// which also takes off the terms of constant zeros that matrix records leave out).  The
+// log's adjoint divides the same way as a body division.
 constexpr double kDivStep = 3, kRcpNewton = 3;
 
 // (the reciprocal of a determinant or pivot is the correctly rounded rcp)

@@ -174,7 +174,7 @@ struct Plan {
   std::vector<double> extra_consts;  // appended after the tape's constant pool
   // algorithmic cost per lane (for the roofline): DFMA-equivalents and saved bytes
   double work_fwd = 0, work_rev = 0;
-  double records_fwd = 0, records_rev = 0;  // to add where compact or matrix records run (their divisions)
+  double records_fwd = 0, records_rev = 0;  // to add where compact or matrix records run
   double n_ops_per_lane = 0;
   // shared per-point values (gradient plans of data-axis tapes): one forward-only plan
   // per region, whose lanes are the points (its parameters are the point's observation

@@ -158,6 +158,12 @@ def test_cost_model_counts(ndvm):
     assert c["work_fwd"] == 3 + 2 * 3 + 1 and c["work_rev"] == 2 * 3 + 2
     c = ndvm.trace_build("(model (params a b) (/ a b))").cost()
     assert c["work_fwd"] == 3 + 3 and c["work_rev"] == 3 + 1
+    # a product with a constant takes the terms of its nonzero elements (4 of 8), a selection none
+    D, S = "(matrix 2 2 1.5 0 0 2.5)", "(matrix 2 2 0 1.0 1.0 0)"
+    for M, terms in ((D, 4), (S, 0), ("(matrix 2 2 1.5 2.0 0.5 2.5)", 8)):
+        c = ndvm.trace_build(f"(model (params a b) (trace (matmul {M} (matrix 2 2 a b b a))))").cost()
+        full = ndvm.trace_build("(model (params a b) (trace (matrix 2 2 a b b a)))").cost()
+        assert c["work_fwd"] - full["work_fwd"] == terms and c["work_rev"] - full["work_rev"] == terms
     lg = ndvm.trace_build(W.logistic(B=1).program, ndvm.FE_BYTECODE)
     assert lg.cost()["spill"] and lg.workspace_bytes(10) == lg.cost()["save_elems"] * 8 * 10
     assert lg.workspace_bytes(10, ndvm.F32) == lg.cost()["save_elems"] * 4 * 10
