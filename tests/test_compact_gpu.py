@@ -3,7 +3,8 @@
 A tape built with NDVM_COMPACT=0 runs on the general kernels.  Both run the same plan; they
 differ in the order in which a data sum's points are added (points per thread) and in
 roundings of the reverse rules that the compact form fuses, so lanes agree within the parity bound
-(1e-12 in binary64, 1e-5 in binary32, of the lane's largest component).  Sizes cover the edges of the split:
+(1e-12 in binary64, 1e-5 in binary32, of the lane's largest component; more only where the oracle's two
+derivative engines disagree by more, as in the parity tests).  Sizes cover the edges of the split:
 fewer points than threads, one more or less than a pass, one lane, ragged warps."""
 import numpy as np
 import pytest
@@ -45,7 +46,7 @@ def test_compact_equals_general(ndvm, oracle_mod, cuda, monkeypatch, B, n, dtype
     f64 = dtype == "float64"
     fast, general = _both(ndvm, w, getattr(torch, dtype), monkeypatch)
     idx = np.unique([0, B // 2, B - 1])
-    ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-12 if f64 else 2e-5)
+    ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-12 if f64 else 1e-5)
     assert ok, rep
     np.testing.assert_array_equal(fast[0], fast[2])  # the value plan's loss is the gradient plan's
     if f64:
@@ -114,15 +115,13 @@ def test_compact_special_values(ndvm, cuda, monkeypatch, n):
     lambda: W.logistic(B=130, n_obs=100, every=10), *[lambda k=k: W.second_client(B=65)[k] for k in range(4)],
     *[lambda k=k: W.control_fuzz(12, B=70, n_points=19, seed=5)[k] for k in range(12)],
     *[lambda k=k: W.random_exprs(8, B=150, n_points=50, seed=3)[k] for k in range(8)]])
-def test_compact_programs(ndvm, cuda, monkeypatch, make, dtype):
+def test_compact_programs(ndvm, oracle_mod, cuda, monkeypatch, make, dtype):
     import torch
     w = make()
     fast, general = _both(ndvm, w, getattr(torch, dtype), monkeypatch)
-    if dtype == "float64":
-        ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-11)
-    else:  # lanes whose gradient nearly cancels differ more: the population's norm
-        rel = np.linalg.norm(fast[1] - general[1]) / max(np.linalg.norm(general[1]), 1e-30)
-        ok, rep = rel < 2e-5 and np.allclose(fast[0], general[0], rtol=2e-5), rel
+    f64 = dtype == "float64"
+    _, _, spread = oracle_ref(oracle_mod, w.program, w.params, w.obs, frontend=w.frontend, f32=not f64)
+    ok, rep = rel_check(fast[0], fast[1], general[0], general[1], 1e-12 if f64 else 1e-5, spread)
     assert ok, rep
 
 

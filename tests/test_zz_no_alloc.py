@@ -30,8 +30,9 @@ def _noalloc(nd, tape, p, o, loss, grad):
 SCRATCH_BYTES = 32 << 20
 
 
-@pytest.mark.parametrize("make", [lambda: W.logistic(B=3000), lambda: W.random_exprs(1, B=3000, n_points=256)[0]],
-                         ids=["workspace-tape", "data-axis-tape"])
+@pytest.mark.parametrize("make", [lambda: W.logistic(B=3000), lambda: W.random_exprs(1, B=3000, n_points=256)[0],
+                                  lambda: W.kalman_cv4(B=3000, T=60), lambda: W.kalman_highd(B=3000, D=20, m=4, T=8)],
+                         ids=["workspace-tape", "data-axis-tape", "matrix-tape", "block-per-lane-tape"])
 def test_noalloc_matches_regular_entry_point_twice(ndvm, cuda, make):
     """Two calls in a row with different inputs and lane counts (3000 lanes; then the last
     1537 lanes with every parameter scaled by 1.05 and the observations by 0.9), each
@@ -39,7 +40,8 @@ def test_noalloc_matches_regular_entry_point_twice(ndvm, cuda, make):
     not read what the first left in the shared scratch.  The logistic tape keeps 4,099
     values per lane, so its 3000 lanes (98 MB) run in more than one launch over the
     32 MiB scratch; the random-expression tape keeps its per-point values shared by all
-    lanes (computed from the observations) at the start of the scratch."""
+    lanes (computed from the observations) at the start of the scratch; the filters are of
+    matrix records, the larger with a block per lane."""
     import torch
     w = make()
     tape = ndvm.trace_build(w.program, w.frontend)
