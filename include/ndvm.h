@@ -138,9 +138,10 @@ size_t ndvm_workspace_bytes_multi(const ndvm_tape* const* tapes, int32_t n_tapes
  * B[k] lanes with its own params[k] (device, B[k] x P_k), obs[k] (device, n_obs[k]
  * values), loss[k] (device, B[k]) and grad[k] (device, B[k] x P_k); the results are
  * those of n_tapes separate ndvm_value_and_grad calls.  Replays of the same kernel
- * variant, block size, threads per lane and occupancy share one launch (up to 240
- * tapes each); a batch with shared per-point values adds one launch of observation
- * copies and one of derive plans in front.
+ * variant, block size and threads per lane share one launch (up to 240 tapes each)
+ * while they have the same occupancy or the launch stays small; a batch with shared
+ * per-point values adds launches of derive plans in front and, for tapes on the
+ * general kernel, one of observation copies.
  *   tapes, B, params, obs, n_obs, loss, grad : host arrays of n_tapes entries
  *   workspace : device, 256-byte aligned, at least ndvm_workspace_bytes_multi bytes
  *               (NULL if that is 0); overwritten; not to be shared with a concurrent call

@@ -449,7 +449,9 @@ bool matrix_shape(const Plan& p, size_t elem, int64_t B, const Shape& g, Shape* 
   // steps, two against two: 1.75 and 2.58; 15 states, 9000 lanes x 6 steps, five against four:
   // 3.43 and 4.00), else twice as many of one, or of two with as many threads per lane (4000
   // lanes x 6 steps of 11 states, two against one: 1.09 ms and 0.89; 16384 lanes x 120 steps of
-  // 8 states, four rounds with 16 threads per lane against two with 8: 19.3 ms and 23.6).
+  // 8 states, four rounds with 16 threads per lane against two with 8: 19.3 ms and 23.6).  Behind
+  // these lines: a round of records takes 0.61 to 0.69 of the general kernel's with as many threads
+  // per lane (the pairs above) and 0.41 with twice as many; they move when a kernel does.
   if (elem == 8 && p.matrix_width >= 128 && 2 * rounds(s) >= 3 * general) return false;
   if (s.log2g >= 3 && rounds(s) >= 2 * general && (general == 1 || (general == 2 && s.log2g == g.log2g))) return false;
   *out = s;

@@ -5,11 +5,10 @@
 // FP64 pipe does only the arithmetic that needs 53-bit precision.
 //
 // exp: table-driven method of P. T. P. Tang (ACM TOMS 15(2), 1989).  x = (64m + j)
-//   ln2/64 + r with |r| <= ln2/128; exp(x) = 2^m 2^(j/64) (1 + p(r)), p the Taylor
-//   polynomial of exp(r) - 1 through r^5 (truncation < 4e-17 relative).  The
-//   nearest integer 64m + j comes from binary32 arithmetic, as does the polynomial's r^4
-//   coefficient; 2^m is applied by an integer add to the exponent field.
-//   7 FP64 instructions (10 with both in binary64, at the same error).
+//   ln2/64 + r; exp(x) = 2^m 2^(j/64) (1 + p(r)), p the Taylor polynomial of exp(r) - 1
+//   through r^5.  The integer 64m + j comes from binary32 arithmetic (nearest below): |r| is up
+//   to 0.507 ln2/64 (truncation < 4e-17 relative).  So does the polynomial's r^4 coefficient;
+//   2^m is applied by an integer add to the exponent field.  7 FP64 instructions (10 with both in binary64, at the same error).
 // log: table-driven method of P. T. P. Tang (ACM TOMS 16(4), 1990).  x = 2^e m with
 //   m in [0.75, 1.5), F = j/128 the nearest table point, f = m - F (exact),
 //   u = f / F by a tabulated reciprocal, log x = e ln2 + ln F + log1p(u) with the
@@ -18,20 +17,21 @@
 //   no cancellation.  11 FP64 instructions (e is converted by integer operations, and the last
 //   coefficient computed in binary32; 13 without, at the same error).
 // sin, cos: additive range reduction of W. J. Cody and W. Waite ("Software Manual for
-//   the Elementary Functions", 1980) by pi/64: x = n pi/64 + r, |r| <= pi/128, with pi/64
+//   the Elementary Functions", 1980) by pi/64: x = n pi/64 + r, |r| <= 0.567 pi/64, with pi/64
 //   in three parts (n times the first two exact for |n| < 2^20), then the addition
 //   formulas over a table of sin(k pi/64), k = n mod 128:
 //   sin x = S + (S (cos r - 1) + C sin r), cos x = C + (C (cos r - 1) - S sin r),
 //   S = sin(k pi/64), C = cos(k pi/64), with sin r through r^7 and cos r - 1 through r^6
-//   (truncation below 4e-19 relative at |r| = pi/128).  No branch on the quadrant: every
-//   lane of a warp runs the same instructions.  14 FP64 instructions for one of them, 17
-//   for both (n by binary32 arithmetic; 16 and 19 without).
+//   (truncation below 1e-18 relative and 9e-18 at the largest |r|; 4e-19 and 4e-18 at pi/128).
+//   No branch on the quadrant: every lane of a warp runs the same instructions.  14 FP64
+//   instructions for one of them, 17 for both (n by binary32 arithmetic; 16 and 19 without).
 // Arguments outside the fast range (|x| >= 708 for exp; x <= 0, subnormal, infinite
 // or NaN for log; |x| >= 2^15, infinite or NaN for sin and cos) take CUDA's functions.
-// Results are within about 1 ulp (sin and cos: 2 ulp, tested).  Against 64-bit mantissas over a
-// million arguments a range, error with the binary32 parts and without them: exp on +-1 1.245
-// ulp at most, rms 0.4104 (1.255, 0.4108); on +-707 1.249, 0.4113 (1.249, 0.4117); log on [0.7, 1.6]
-// 1.519, 0.4363 both ways; sin on +-1000 1.768, 0.3941 both ways.
+// Results are within 1.3 ulp (exp), 1.6 (log) and 2.1 (sin, cos; 2 tested).  Against 64-bit mantissas
+// over 40 million arguments a range, largest error in ulp and rms with the binary32 parts and
+// without them: exp on +-707 1.281, 0.4113 (1.274, 0.4117); log on [0.7, 1.6] 1.590, 0.4363 both ways;
+// sin on +-10 1.563, 0.3918 both ways, on +-32767 1.989, 0.3943 (1.989, 0.3944); cos there 2.071,
+// 0.3945 both ways.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -76,7 +76,10 @@ __device__ __forceinline__ double to_f64(float x) {
   return __hiloint2double((int)hi, (int)(b << 29));
 }
 
-// the integer nearest to x * scale (within 2^-20 of a tie either one), in binary32
+// an integer near x * scale, in binary32: x is cut to 24 bits and the product's factor rounded, so
+// it may be a neighbour of the nearest one, the farther the larger |x|: at most 0.507 from
+// x * scale for exp's arguments, 0.503 for those of sin and cos up to 1000 and 0.567 up to 2^15
+// (half a unit, plus x * scale times the 2^-23 cut off and the scale's error)
 __device__ __forceinline__ float nearest(double x, float scale) { return fmaf(to_f32(x), scale, 12582912.0f); }
 __device__ __forceinline__ int nearest_int(float t) { return (int)__float_as_uint(t) - 0x4b400000; }
 __device__ __forceinline__ double nearest_f64(float t) { return to_f64(t - 12582912.0f); }

@@ -355,7 +355,7 @@ void Planner::analyze() {
           // the reverse rule reads b and, inside a data-axis body (where it stays in a slot
           // for the point's reverse sweep), the forward sweep's reciprocal of b; a lane-level
           // division divides again (a workspace round trip for the reciprocal measured no
-          // faster on a serial chain)
+          // faster on a serial chain of the general kernel; compact streams may share one)
           need(n.b); if (active_[n.b]) need(v);
           if (region_body_[v]) need_aux_[v] = 1;
           break;
